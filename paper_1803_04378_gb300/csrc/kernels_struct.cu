@@ -39,7 +39,7 @@
 // structure-aware rebuild; k_struct_layout / k_struct_gather_* then gather the
 // live columns of the rebuilt B^-1 into bp.
 #include "lpgb_internal.cuh"
-#include "iter_common.cuh"
+#include "struct_common.cuh"
 #include "../../include/lpgb.h"
 
 #include <cfloat>
@@ -47,61 +47,6 @@
 namespace lpgb {
 
 namespace {
-
-// The slot moves of one pivot (every CTA computes the same values).
-struct SlotMoves {
-    int join, ent;   // rows entering / leaving R (-1: none)
-    int k0, k1, kn;  // live slots before, after the join, after the drop
-    int tl;          // old slot of `join`
-    int u;           // row displaced from slot k0 by the join
-    int te;          // slot of `ent`, which receives row w
-    int w;           // row moved into slot te
-    int J;           // new slot of the joining row's column (-1: none)
-    int src_te;      // old slot whose column moves to te (-1: none or the join)
-};
-
-__device__ SlotMoves slot_moves(const DevState& s, int leave, int q, int k, int par) {
-    const Params& P = s.p;
-    const int32_t* sr = s.slot_row + (size_t)par * P.m;
-    const int32_t* rs = s.row_slot + (size_t)par * P.m;
-    SlotMoves v;
-    v.join = leave >= P.n ? leave - P.n : -1;
-    v.ent = q >= P.n ? q - P.n : -1;
-    v.k0 = k;
-    v.tl = v.join >= 0 ? __ldcg(rs + v.join) : -1;
-    v.u = v.join >= 0 ? __ldcg(sr + k) : -1;
-    v.k1 = k + (v.join >= 0 ? 1 : 0);
-    v.te = v.ent >= 0 ? __ldcg(rs + v.ent) : -1;
-    v.w = v.ent >= 0 ? (v.join >= 0 ? v.join : __ldcg(sr + k - 1)) : -1;
-    v.kn = v.k1 - (v.ent >= 0 ? 1 : 0);
-    v.J = v.join >= 0 ? (v.ent >= 0 ? v.te : v.k0) : -1;
-    v.src_te = (v.ent >= 0 && v.join < 0) ? v.k0 - 1 : -1;
-    return v;
-}
-
-// new slot_row entry of slot t / new row_slot entry of row x
-__device__ __forceinline__ int moved_slot_row(const SlotMoves& v, int t, int old) {
-    if (v.ent >= 0 && t == v.te) return v.w;
-    if (v.ent >= 0 && t == v.k1 - 1) return v.ent;
-    if (v.join >= 0 && t == v.k0) return v.join;
-    if (v.join >= 0 && t == v.tl) return v.u;
-    return old;
-}
-__device__ __forceinline__ int moved_row_slot(const SlotMoves& v, int x, int old) {
-    if (v.ent >= 0 && x == v.ent) return v.k1 - 1;
-    if (v.ent >= 0 && x == v.w) return v.te;
-    if (v.join >= 0 && x == v.join) return v.J;
-    if (v.join >= 0 && x == v.u) return v.tl;
-    return old;
-}
-
-// Source of slot t's rho and y after the moves: an old slot, or -2 for the
-// joining row (rho = 1, y = 0: its old column is e_r and its y is zero).
-__device__ __forceinline__ int vec_src(const SlotMoves& v, int t) {
-    if (t == v.J) return -2;
-    if (t == v.te && v.src_te >= 0) return v.src_te;
-    return t;
-}
 
 constexpr int kMaxOwnedRows = 256;  // rows of B^-1 per CTA (ratio-test records kept in shared memory)
 
@@ -115,38 +60,6 @@ constexpr int kMaxOwnedRows = 256;  // rows of B^-1 per CTA (ratio-test records 
 // kn.  Row l of the CTA leaves alpha', bbar_i and its basic variable in
 // ral/rb/rvar[l] (alpha' and the variable also in global memory for the ratio
 // test of other CTAs); the ratios themselves are formed in row_record.
-// Warp sum of a + b over the 32 lanes (every lane gets it) in 64-bit fixed
-// point.  The values are aligned to the warp's largest binary exponent E
-// (one redux): a value is t 2^(E - 1079) with |t| < 2^57, rounded to nearest;
-// the t are added exactly by integer shuffles, and the sum is rounded to
-// binary64 once (ll_scaled).  Relative to 2^(E - 1022), which bounds every
-// |value|, the error is below 2^-51 plus the final rounding -- no more than
-// the FP64 butterfly's -- and the sum does not depend on the lane order.  It
-// spends no FP64 instruction (each holds the FP64 pipe for ~64 cycles on this
-// chip, and the butterfly needs six per row).  Subnormal, infinite and NaN
-// inputs take the FP64 butterfly.
-__device__ __forceinline__ double warp_sum2_fixed(double a, double b) {
-    const unsigned long long ua = (unsigned long long)__double_as_longlong(a);
-    const unsigned long long ub = (unsigned long long)__double_as_longlong(b);
-    const int ea = (int)((ua >> 52) & 0x7ff), eb = (int)((ub >> 52) & 0x7ff);
-    const bool odd = (ea == 0 && (ua << 1) != 0) || (eb == 0 && (ub << 1) != 0) || ea == 0x7ff || eb == 0x7ff;
-    const unsigned emax = __reduce_max_sync(0xffffffffu, (unsigned)max(ea, eb));
-    if (__any_sync(0xffffffffu, odd) || emax == 0) return warp_sum(a + b);
-    auto fix = [emax](unsigned long long u, int e) -> long long {
-        if (e == 0) return 0;  // +-0
-        const long long mant = (long long)((u & 0xFFFFFFFFFFFFFull) | (1ull << 52));
-        const int sh = e - (int)emax + 4;  // at most 4
-        long long t = 0;
-        if (sh >= 0) t = mant << sh;
-        else if (sh > -60) t = (mant + (1ll << (-sh - 1))) >> (-sh);
-        return (u >> 63) ? -t : t;
-    };
-    long long t = fix(ua, ea) + fix(ub, eb);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    return t == 0 ? 0.0 : ll_scaled(t, (int)emax - 1079);
-}
-
 // upd: which rows take the pending rank-1 update here -- kUpdAll, kUpdRowR
 // (only row r: the others were updated by the update warps while the rest of
 // the CTA priced), kUpdButR (every row but r, no FTRAN: the update warps), or
@@ -238,68 +151,6 @@ __device__ void update_block_s(const DevState& s, const SlotMoves& v, int r, int
                 rvar[l] = var;
             }
         }
-    }
-}
-
-// The CTA's ratio-test record from its rows' (alpha', bbar, variable): its
-// smallest ratio, and its best row and tie count under that ratio's tie
-// threshold (one warp, one lane per row).  On this chip every FP64
-// instruction holds a scheduler's FP64 pipe for 64 cycles whatever the number
-// of active lanes, so the ratios of 32 rows are formed by one warp-wide
-// division; the minimum, the tie band and the largest pivot are taken on
-// integer keys, across the warp by redux (a dependent shuffle costs more).
-__device__ void row_record(const Params& P, int owned, bool bland, const double* ral, const double* rb,
-                           const int* rvar, RowRec* out) {
-    const int lane = threadIdx.x & 31;
-    const int G = gridDim.x;
-    const long long kpiv = dkey(P.tol_piv), kbig = dkey(DBL_MAX);
-    // pass 1: ratios and their minimum
-    long long kmin_l = kbig;
-    double th0 = DBL_MAX;  // the first 32 rows' ratios, kept for pass 2
-    for (int l0 = 0; l0 < owned; l0 += 32) {
-        const int l = l0 + lane;
-        const double al = l < owned ? ral[l] : 0.0;
-        const bool ok = l < owned && dkey(al) > kpiv;
-        const double th = ok ? rb[l] / al : DBL_MAX;
-        if (l0 == 0) th0 = th;
-        kmin_l = min(kmin_l, dkey(th));
-    }
-    const long long kmin = warp_min_key(kmin_l);
-    const double tmin = kdouble(kmin);
-    const double thr = kmin == kbig ? DBL_MAX : tmin + P.tol_tie * fmax(1.0, fabs(tmin));
-    const long long kthr = dkey(thr);
-    // pass 2: the tie band, its size and best row (largest pivot, then smallest
-    // basic index; Bland: smallest basic index), lane by lane
-    long long ka = LLONG_MIN;
-    int bvar = INT_MAX, bl = -1, cnt = 0;
-    double bth = 0.0;
-    if (kmin != kbig) {
-        for (int l0 = 0; l0 < owned; l0 += 32) {
-            const int l = l0 + lane;
-            const double al = l < owned ? ral[l] : 0.0;
-            const long long kal = dkey(al);
-            const bool ok = l < owned && kal > kpiv;
-            const double th = l0 == 0 ? th0 : (ok ? rb[l] / al : DBL_MAX);
-            if (ok && dkey(th) <= kthr) {
-                cnt++;
-                const int v = rvar[l];
-                const bool better = bl < 0 || (bland ? v < bvar : (kal > ka || (kal == ka && v < bvar)));
-                if (better) { ka = kal; bvar = v; bl = l; bth = th; }
-            }
-        }
-    }
-    const int tot = __reduce_add_sync(0xffffffffu, cnt);
-    long long kbest;
-    const int win = bland ? warp_argmin_index(bvar, bl >= 0)
-                          : warp_argmax_key(ka, bvar, bl >= 0, kbest);
-    if (win < 0 ? lane == 0 : lane == win) {
-        RowRec rp;
-        rp.tmin = kmin; rp.thr = kthr;
-        rp.a = win >= 0 ? kdouble(ka) : 0.0;
-        rp.th = win >= 0 ? bth : 0.0;
-        rp.var = win >= 0 ? bvar : 0; rp.row = win >= 0 ? (int)blockIdx.x + G * bl : -1;
-        rp.cnt = tot; rp.pad_ = 0;
-        *out = rp;
     }
 }
 
@@ -482,24 +333,6 @@ __device__ Cand reduce_price_parts_s(const PriceRec* part, int nparts, bool need
     return g;
 }
 
-__device__ PricePatch pivot_patch(const SlotMoves& v, int q, int leave, bool push, int tabu_until) {
-    PricePatch p = no_patch();
-    p.basic_j = q;
-    p.free_j = leave;
-    if (push) { p.tabu_j = leave; p.tabu_until = tabu_until; }
-    // the slot -> row entries that differ from the current map, in the
-    // precedence order of moved_slot_row
-    if (v.ent >= 0) {
-        p.sp_slot[p.nsp] = v.te; p.sp_row[p.nsp] = v.w; ++p.nsp;
-        p.sp_slot[p.nsp] = v.k1 - 1; p.sp_row[p.nsp] = v.ent; ++p.nsp;
-    }
-    if (v.join >= 0) {
-        p.sp_slot[p.nsp] = v.k0; p.sp_row[p.nsp] = v.join; ++p.nsp;
-        p.sp_slot[p.nsp] = v.tl; p.sp_row[p.nsp] = v.u; ++p.nsp;
-    }
-    return p;
-}
-
 // One step = apply the pivot chosen by the last ratio test and price (A),
 // grid barrier, CHUZC + UPDATE/FTRAN + the CTA's ratio-test record (B), grid
 // barrier, CHUZR (C).  Step (A) needs no barrier of its own: every CTA
@@ -534,13 +367,6 @@ __device__ PricePatch pivot_patch(const SlotMoves& v, int q, int leave, bool pus
 // smallest-index rule of the safety net needs every improving column, so
 // under it the full FP64 PRICE runs.
 constexpr int kScreenMaxList = kPriceThreads;
-
-// order-preserving integer image of a float (no NaN; -0 and +0 share one key)
-__device__ __forceinline__ int fkey(float x) {
-    int b = __float_as_int(x);
-    if ((b & 0x7fffffff) == 0) b = 0;
-    return b >= 0 ? b : (b ^ 0x7fffffff);
-}
 
 // kNC columns at once: s[c] = sum y a_c and a[c] = sum |y| |a_c| over the n4
 // float4 groups, lane-strided, then across the warp by butterflies (every lane
@@ -894,7 +720,10 @@ __global__ void __launch_bounds__(kUpdateThreads, 1) k_iterate_s(DevState s, int
         }
         if (threadIdx.x == 0) {
             if (piv) {
-                mv = slot_moves(s, S.leave, S.q, S.k, par);
+                const int32_t* sr0 = s.slot_row + (size_t)par * P.m;
+                const int32_t* rs0 = s.row_slot + (size_t)par * P.m;
+                mv = slot_moves(P.n, S.leave, S.q, S.k, [rs0](int x) { return __ldcg(rs0 + x); },
+                                [sr0](int t) { return __ldcg(sr0 + t); });
                 const bool degenerate = th <= P.tol_tie;
                 const bool push = P.tabu_tenure > 0 && (S.tcount > 1 || degenerate);
                 ppat = pivot_patch(mv, S.q, S.leave, push, S.it + 1 + P.tabu_tenure);
@@ -974,17 +803,8 @@ __global__ void __launch_bounds__(kUpdateThreads, 1) k_iterate_s(DevState s, int
             }
             if (mv.join >= 0 || mv.ent >= 0) {
                 // A_p rows of the columns this CTA prices follow their slots
-                int dst[3], src[3], nm = 0;
-                if (mv.ent >= 0 && mv.join >= 0) {
-                    dst[0] = mv.te; src[0] = mv.tl;
-                    dst[1] = mv.k0; src[1] = mv.te;
-                    nm = 2;
-                    if (mv.tl != mv.k0) { dst[2] = mv.tl; src[2] = mv.k0; nm = 3; }
-                } else if (mv.ent >= 0) {
-                    if (mv.te != mv.k0 - 1) { dst[0] = mv.te; src[0] = mv.k0 - 1; dst[1] = mv.k0 - 1; src[1] = mv.te; nm = 2; }
-                } else if (mv.tl != mv.k0) {
-                    dst[0] = mv.k0; src[0] = mv.tl; dst[1] = mv.tl; src[1] = mv.k0; nm = 2;
-                }
+                int dst[3], src[3];
+                const int nm = slot_row_moves(mv, dst, src);
                 for (int j = blockIdx.x + G * threadIdx.x; j < P.n && nm > 0; j += G * blockDim.x) {
                     double* col = s.A_p + (size_t)j * P.ld;
                     float* col32 = s.A_p32 + (size_t)j * P.ld;

@@ -294,6 +294,21 @@ bool struct_engine_fits(int m, int ld, int ctas);  // shared-memory and per-CTA 
 void launch_struct_enter(const DevState& s, int force, int32_t* relayout, cudaStream_t st, bool compact);
 void launch_struct_scatter_y(const DevState& s, cudaStream_t st);  // yp -> y (row order)
 void launch_struct_init_maps(const DevState& s, cudaStream_t st);
+// The same with the working set in shared memory (kernels_resident.cu).
+struct ResidentPlan {
+    int ctas;      // CTAs of the launch
+    int kc;        // live slots the layout holds
+    bool a, b;     // the FP32 copy of A, the rows of B^-1 in shared memory
+    size_t smem;
+};
+int resident_ctas(int sms, int m, int n);
+size_t resident_meet_bytes(int ctas);  // the CTAs' records (zero before the first launch)
+// false: not even the vectors fit
+bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t smem_optin, ResidentPlan* out);
+// uses the meeting numbers seq0 + 1 .. seq0 + resident_meetings(iters)
+inline unsigned resident_meetings(int iters) { return 4u * (unsigned)iters + 2u; }
+cudaError_t launch_iterate_r(const DevState& s, const ResidentPlan& p, int iters, void* meet, unsigned seq0,
+                             cudaStream_t st);
 // Bounded-wait self-test: a grid barrier that cannot complete (lp_selftest_barrier_timeout).
 int barrier_selftest(int blocks, cudaStream_t st);
 size_t price_smem_bytes(int ld);

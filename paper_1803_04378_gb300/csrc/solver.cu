@@ -71,6 +71,10 @@ struct lp_handle {
                                      // B^-1 and y are stale while it is
     bool s_force = true;             // rebuild the slot map and A_p on the next entry
     int32_t* s_relayout = nullptr;   // device flag: the entry rebuilt the slot map
+    int r_ctas = 0;                  // k_iterate_r: CTAs per launch
+    size_t smem_optin = 0;           // shared memory a block may use
+    ulonglong2* r_meet = nullptr;    // k_iterate_r: the CTAs' records
+    unsigned r_seq = 0;              // last meeting number handed out
     int32_t* csc_cnt = nullptr;      // price_mode 2: per-column nonzero counts (scratch)
     double chain_s = 0.0, chain_b = 0.0;
     int chain_n = 0;
@@ -494,6 +498,21 @@ int reinvert(lp_handle* h, int check_feasible, bool refine, bool to_struct = fal
     if (redo) return reinvert(h, check_feasible, false, to_struct);
     if (q.compact) TRY(struct_enter_compact(h));
     return LP_OK;
+}
+
+// Up to graph_iters + 1 steps of the structured engine: the resident kernel
+// where its vectors fit in shared memory, else (and for the lexicographic rule
+// and a priority list, which it does not have) k_iterate_s.
+cudaError_t launch_structured(lp_handle* h, int k_live) {
+    const int iters = h->opt.graph_iters + 1;
+    ResidentPlan rp;
+    if (!h->p.lex && !h->p.prio &&
+        resident_plan(h->m, h->n, h->ld, h->r_ctas, k_live, iters, h->smem_optin, &rp)) {
+        const unsigned seq0 = h->r_seq;
+        h->r_seq += resident_meetings(iters);
+        return launch_iterate_r(h->ds, rp, iters, h->r_meet, seq0, h->stream);
+    }
+    return launch_iterate_s(h->ds, h->persist_blocks, iters, h->stream);
 }
 
 int reset_state(lp_handle* h) {
@@ -969,6 +988,12 @@ static int create_impl(lp_handle* h, int32_t m, int32_t n, const double* A, cons
             TRY(dalloc(h, &h->s_relayout, 1));
             TRY(dalloc(h, &s.price_rec, (size_t)h->geo.sms));
             TRY(dalloc(h, &s.row_rec, (size_t)h->geo.sms));
+            int optin = 0;
+            CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
+            h->smem_optin = (size_t)optin;
+            h->r_ctas = resident_ctas(h->geo.sms, m, n);
+            TRY(dalloc(h, &h->r_meet, resident_meet_bytes(h->r_ctas) / sizeof(ulonglong2)));
+            CK(cudaMemsetAsync(h->r_meet, 0, resident_meet_bytes(h->r_ctas), h->stream));
             CK(cudaMemsetAsync(s.bp, 0, sizeof(double) * (size_t)m * ld, h->stream));
             CK(cudaMemsetAsync(s.yp, 0, sizeof(double) * 2 * (size_t)ld, h->stream));
             launch_struct_init_maps(s, h->stream);
@@ -1255,7 +1280,7 @@ int lp_solve(lp_handle* h, lp_result* out) {
             if (h->evc0) CK(cudaEventRecord(h->evc0, h->stream));
             // one step more than graph_iters: the first step after an entry only
             // prices and runs the ratio test, so a reinversion period fits one launch
-            const cudaError_t e = launch_iterate_s(h->ds, h->persist_blocks, h->opt.graph_iters + 1, h->stream);
+            const cudaError_t e = launch_structured(h, C.k_live);
             if (e == cudaSuccess) {
                 h->launches += 1;
                 if (h->evc1) CK(cudaEventRecord(h->evc1, h->stream));
