@@ -464,8 +464,9 @@ int lp_batch_get_trace(const lp_batch* h, int32_t k, int32_t* q, int32_t* r, int
 
 /*
  * Autotuner.  table[2*b] = threads per CTA (128, 256 or 512) and
- * table[2*b+1] = 1 to keep B^-1 in shared memory (only where it fits) or 0
- * for an L2-resident global slot, for size buckets b = 0..3.
+ * table[2*b+1] = 1 to keep the first live columns of B^-1 in shared memory (only
+ * for buckets whose whole inverse would fit) or 0 for an L2-resident global
+ * slot, for size buckets b = 0..3.
  * lp_batch_tune times every valid configuration of every non-empty bucket on
  * the batch itself (`trials` solves each), keeps the fastest, and writes the
  * table if it is not NULL; lp_batch_set_tuning installs a saved table.

@@ -17,8 +17,9 @@
 // PRICE runs whenever no candidate improves or Bland's rule is on.  FTRAN, the
 // ratio test, the B^-1 update and reinversion are FP64.
 //
-// B^-1 is stored column-major (element (i, k) at Binv[k*m + i]) so that a
-// thread per row reads consecutive addresses in FTRAN.
+// B^-1 is kept in slack-structured form: only the columns of rows whose slack is
+// nonbasic, column-major, so that a thread per row reads consecutive addresses.
+#include "iter_common.cuh"
 #include "lpgb_internal.cuh"
 #include "../../include/lpgb.h"
 
@@ -71,213 +72,72 @@ constexpr int kBatchMaxM = 256;
 constexpr int kBatchMaxN = 512;
 constexpr int kBatchTopk = 8;
 constexpr int kSlotsPerSm = 8;  // scratch slots per SM and bucket (CTAs per SM at most)
+constexpr int kSmemCols = 16;   // live columns of B^-1 in shared memory where the tuning asks for it
 
 namespace {
 
-// ---------------------------------------------------------------- reductions
-// Values are ordered through their integer images (dkey): every FP64 compare
-// or min would hold the FP64 pipe as long as an FMA on this chip.
-struct BCand { long long d; int j; };  // d: dkey image
-
-__device__ __forceinline__ bool bc_beats(long long da, int ja, long long db, int jb) {
-    if (ja < 0) return false;
-    if (jb < 0) return true;
-    return da > db || (da == db && ja < jb);
-}
-
-// Block argmax of (d, j) with exact ties to the smallest j; result broadcast.
-template <int T>
-__device__ BCand block_best(BCand c, BCand* sh) {
-    for (int o = 16; o > 0; o >>= 1) {
-        BCand x;
-        x.d = __shfl_xor_sync(0xffffffffu, c.d, o);
-        x.j = __shfl_xor_sync(0xffffffffu, c.j, o);
-        if (bc_beats(x.d, x.j, c.d, c.j)) c = x;
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[w] = c;
-    __syncthreads();
-    BCand r = sh[0];
-    for (int i = 1; i < T / 32; ++i)
-        if (bc_beats(sh[i].d, sh[i].j, r.d, r.j)) r = sh[i];
-    __syncthreads();
-    return r;
-}
-
-template <int T>
-__device__ int block_sum_int(int v, int* sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    int r = 0;
-    for (int i = 0; i < T / 32; ++i) r += sh[i];
-    __syncthreads();
-    return r;
-}
-
-// Block minimum of dkey images; thread 0 also forms the ratio test's tie
-// threshold of the minimum (one FP64 evaluation per block), broadcast in *thr.
-template <int T>
-__device__ long long block_min_key(long long v, long long* sh, double tol_tie, long long* thr) {
-    for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    long long r = sh[0];
-    for (int i = 1; i < T / 32; ++i) r = min(r, sh[i]);
-    if (threadIdx.x == 0) {
-        const double t = kdouble(r);
-        *thr = t == DBL_MAX ? r : dkey(t + tol_tie * fmax(1.0, fabs(t)));
-    }
-    __syncthreads();
-    return r;
-}
-
-template <int T>
-__device__ double block_sum(double v, double* sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    double r = 0.0;
-    for (int i = 0; i < T / 32; ++i) r += sh[i];
-    __syncthreads();
-    return r;
-}
-
-// Leaving-row candidate: largest alpha, ties to the smallest basic variable
-// (Bland: smallest basic variable).
-struct RCand { long long a; int var; int row; };  // a: dkey image of alpha
-
-__device__ __forceinline__ bool rc_beats(const RCand& x, const RCand& y, bool bland) {
-    if (x.row < 0) return false;
-    if (y.row < 0) return true;
-    if (bland) return x.var < y.var;
-    return x.a > y.a || (x.a == y.a && x.var < y.var);
-}
-
-template <int T>
-__device__ RCand block_row(RCand c, bool bland, RCand* sh, int& cnt, int* shc) {
-    for (int o = 16; o > 0; o >>= 1) {
-        RCand x;
-        x.a = __shfl_xor_sync(0xffffffffu, c.a, o);
-        x.var = __shfl_xor_sync(0xffffffffu, c.var, o);
-        x.row = __shfl_xor_sync(0xffffffffu, c.row, o);
-        if (rc_beats(x, c, bland)) c = x;
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) { sh[w] = c; shc[w] = cnt; }
-    __syncthreads();
-    RCand r = sh[0];
-    int total = shc[0];
-    for (int i = 1; i < T / 32; ++i) {
-        if (rc_beats(sh[i], r, bland)) r = sh[i];
-        total += shc[i];
-    }
-    __syncthreads();
-    cnt = total;
-    return r;
-}
-
 __device__ __forceinline__ float bf16f(uint16_t v) { return __uint_as_float((uint32_t)v << 16); }
 
-// Scalars of the LP being solved (shared memory).
+// order-preserving integer image of a float (no NaN; -0 and +0 share one key)
+__device__ __forceinline__ int fkey(float x) {
+    int b = __float_as_int(x);
+    if ((b & 0x7fffffff) == 0) b = 0;
+    return b >= 0 ? b : (b ^ 0x7fffffff);
+}
+
+// Scalars of the LP being solved and the block's reduction scratch (shared memory).
 struct LPScal {
-    int status, it, q, r, tcount, degen_run, bland, flags, k, err;
-    double dq, theta, z;
+    int status, it, degen_run, bland, flags, k, err;
+    double z;
 };
-
 struct Red {
-    BCand bc[32];
-    RCand rc[32];
-    double dv[32];
-    long long kv[33];  // keys; kv[32]: the tie threshold
-    int iv[32];
-    int kj[16 * kBatchTopk];   // top-K selection: each warp's kept columns
-    float kd[16 * kBatchTopk];
+    int gmax[32];              // screen: the largest key of each lane's columns over all warps
+    int lcount, lkey[32], lj[32];  // columns at or above the top-K threshold
+    int sel[16][kBatchTopk];   // per warp: the top K of the list, best first
+    double cd[kBatchTopk];     // their exact reduced costs
+    int cj[kBatchTopk];
+    long long wk[16];          // per warp: a key,
+    int wj[16], wv[16], wc[16];  // an index, a variable, a count
+    double wa[16], wt[16];
+    double dq;
 };
 
-// ---------------------------------------------------------------- one LP
-// Top K (K <= kBatchTopk) screened columns, best first, in the order
-// (larger d, then smaller j); entries of -FLT_MAX are not candidates.  Each
-// warp ranks its columns among themselves by counting the columns that beat
-// them (no barrier), keeps ranks below K, and warp 0 ranks the kept columns of
-// all warps the same way: cand[t] is the t-th best (-1 when fewer exist).
+// Argmax of (key, j) over the block's valid candidates, exact ties to the smallest j
+// (j = -1 when there is none); every thread gets the result.
 template <int T>
-__device__ void batch_topk(const float* dts, int n, int K, int* cand, int* kj, float* kd) {
-    constexpr int W = T / 32;
-    constexpr int V = (kBatchMaxN + T - 1) / T;  // columns per lane
+__device__ __forceinline__ void block_best(long long key, int j, Red& R, long long& kbest, int& jbest) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    auto beats = [](float da, int ja, float db, int jb) { return da > db || (da == db && ja < jb); };
-    float d[V];
-    int j[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-        j[v] = (int)threadIdx.x + T * v;
-        d[v] = j[v] < n ? dts[j[v]] : -FLT_MAX;
-        if (d[v] == -FLT_MAX) j[v] = -1;
-    }
-    if (lane < K) kj[w * K + lane] = -1;
-    __syncwarp();
-    int rank[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) rank[v] = 0;
-    for (int src = 0; src < 32; ++src) {
-#pragma unroll
-        for (int u = 0; u < V; ++u) {
-            const float od = __shfl_sync(0xffffffffu, d[u], src);
-            const int oj = __shfl_sync(0xffffffffu, j[u], src);
-#pragma unroll
-            for (int v = 0; v < V; ++v)
-                if (oj >= 0 && j[v] >= 0 && beats(od, oj, d[v], j[v])) rank[v]++;
-        }
-    }
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-        if (j[v] >= 0 && rank[v] < K) {
-            kj[w * K + rank[v]] = j[v];
-            kd[w * K + rank[v]] = d[v];
-        }
+    long long kb;
+    const int win = warp_argmax_key(key, j, j >= 0, kb);
+    if (lane == (win < 0 ? 0 : win)) { R.wk[w] = kb; R.wj[w] = win < 0 ? -1 : j; }
     __syncthreads();
-    if (w == 0) {
-        constexpr int C = (W * kBatchTopk + 31) / 32;  // kept columns per lane
-        float cd[C];
-        int cj[C], cr[C];
+    kbest = R.wk[0];
+    jbest = R.wj[0];
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const int e = lane + 32 * c;
-            cj[c] = e < W * K ? kj[e] : -1;
-            cd[c] = cj[c] >= 0 ? kd[e] : -FLT_MAX;
-            cr[c] = 0;
-        }
-        for (int src = 0; src < 32; ++src) {
-#pragma unroll
-            for (int u = 0; u < C; ++u) {
-                const float od = __shfl_sync(0xffffffffu, cd[u], src);
-                const int oj = __shfl_sync(0xffffffffu, cj[u], src);
-#pragma unroll
-                for (int c = 0; c < C; ++c)
-                    if (oj >= 0 && cj[c] >= 0 && beats(od, oj, cd[c], cj[c])) cr[c]++;
-            }
-        }
-        if (lane < K) cand[lane] = -1;
-        __syncwarp();
-#pragma unroll
-        for (int c = 0; c < C; ++c)
-            if (cj[c] >= 0 && cr[c] < K) cand[cr[c]] = cj[c];
-    }
+    for (int i = 1; i < T / 32; ++i)
+        if (beats(R.wk[i], R.wj[i], kbest, jbest)) { kbest = R.wk[i]; jbest = R.wj[i]; }
     __syncthreads();
 }
 
-template <int T, bool SMEM>
-__device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, double* slot, int mmax, int nmax) {
+// ---------------------------------------------------------------- one LP
+// The method on the slack-structured inverse (kernels_struct.cu): only the k columns
+// of B^-1 that belong to rows with a nonbasic slack differ from unit columns and
+// only their duals from zero, so PRICE, FTRAN and the update work on k rows or
+// columns and the slack basis needs no initialisation.  The batch's LPs end
+// after 30 pivots on average, so k is far below m.
+//
+// Threads own rows (i = tid, tid + T, ..) through FTRAN, the ratio test and the update
+// -- alpha, the ratio and the row's entries never leave the thread -- and columns
+// (j = tid, tid + T, ..) through the screen, which then reads a live row of A
+// coalesced.  Live column t lies in shared memory for t < ks, else in the CTA's
+// L2-resident slot.
+//
+// What bounds it: the FP64 pipe (2 k m FMAs and m divisions a pivot, about 4 us of an
+// SM at m = 225, k = 25; 65% of the time on 4096 LPs) and, with few LPs, the latency of
+// a pivot (7.8 us at m <= 128).  Against the dense m x m inverse: 4096 LPs
+// of m 16..256 30.6 -> 3.3 ms, 48 LPs of m 16..128 1.04 -> 0.39 ms, the same pivots.
+template <int T>
+__device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, double* slot, int mmax, int nmax, int ks) {
     const BatchParams& P = s.p;
     const BatchLP L = s.lps[lp];
     const int m = L.m, n = L.n, N = n + m;
@@ -285,393 +145,485 @@ __device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, doub
     const uint16_t* Alp = s.A_lp ? s.A_lp + L.a_off : nullptr;
     const double* b = s.b + L.r_off;
     const double* c = s.c + L.c_off;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int W = T / 32;
+    constexpr int VR = (kBatchMaxM + T - 1) / T;  // rows and columns per thread
+    constexpr int VC = (kBatchMaxN + T - 1) / T;
 
-    // shared-memory carve-up (sizes by the bucket maximum)
-    double* dp = reinterpret_cast<double*>(smem);
-    double* Binv;
-    if (SMEM) { Binv = dp; dp += (size_t)mmax * mmax; }
-    else { Binv = slot; slot += (size_t)mmax * mmax; }
-    double* W = slot;  // reinversion block, k x k column-major (global slot)
-    double* y = dp; dp += mmax;
+    // shared-memory carve-up (sizes by the bucket's largest LP)
+    double* cs = reinterpret_cast<double*>(smem);  // live columns 0 .. ks - 1
+    double* dp = cs + (size_t)ks * mmax;
+    double* y = dp; dp += mmax;      // duals of the live rows, slot order
+    double* rho = dp; dp += mmax;    // rho / alpha_r, slot order
+    double* aq = dp; dp += mmax;     // the entering column on the live rows, slot order
+    double* au = dp; dp += mmax;     // and on the row of position i's basic slack (zero: structural)
     double* bbar = dp; dp += mmax;
-    double* al = dp; dp += mmax;
-    double* rho = dp; dp += mmax;
-    double* aq = dp; dp += mmax;
-    double* th = dp; dp += mmax;
     float* y32 = reinterpret_cast<float*>(dp);
-    float* dts = y32 + mmax;                       // nmax screened values
-    int* ip = reinterpret_cast<int*>(dts + nmax);
-    int* basis = ip; ip += mmax;
-    int* pos = ip; ip += nmax + mmax;
-    int* tabu = ip; ip += nmax + mmax;
-    int* lstP = ip; ip += mmax;
-    int* lstR = ip; ip += mmax;
-    int* pivrow = ip; ip += mmax;
-    int* pinv = ip; ip += mmax;
-    int* cand = ip; ip += kBatchTopk + 1;
-    double* cand_d = reinterpret_cast<double*>(((uintptr_t)ip + 7) & ~(uintptr_t)7);
+    float* cf = y32 + mmax;
+    int* tabu = reinterpret_cast<int*>(cf + nmax);
+    int16_t* basis = reinterpret_cast<int16_t*>(tabu + nmax + mmax);
+    int16_t* pos = basis + mmax;
+    int16_t* srow = pos + nmax + mmax;   // slot -> row
+    int16_t* rslot = srow + mmax;        // row -> slot, -1: basic slack
+    int16_t* lstP = rslot + mmax;
+    int16_t* lstR = lstP + mmax;
+    int16_t* pivrow = lstR + mmax;
+    int16_t* pinv = pivrow + mmax;
+    double* gcol = slot;                              // live columns ks ..
+    double* Wm = slot + (size_t)mmax * mmax;          // reinversion block, k x k column-major
+    auto col = [&](int t) -> double* { return t < ks ? cs + (size_t)t * m : gcol + (size_t)(t - ks) * m; };
 
     __shared__ LPScal S;
     __shared__ Red R;
+    const long long ktol = dkey(P.tol_d), kpiv = dkey(P.tol_piv), kbig = dkey(DBL_MAX);
 
     // Step 1: slack basis
-    for (int e = tid; e < m * m; e += T) Binv[e] = (e / m == e % m) ? 1.0 : 0.0;
     for (int i = tid; i < m; i += T) {
-        y[i] = 0.0;
-        y32[i] = 0.f;
         bbar[i] = b[i];
-        basis[i] = n + i;
+        basis[i] = (int16_t)(n + i);
+        rslot[i] = -1;
+        au[i] = 0.0;
     }
     for (int j = tid; j < N; j += T) {
-        pos[j] = j < n ? -1 : j - n;
+        pos[j] = (int16_t)(j < n ? -1 : j - n);
         tabu[j] = 0;
+        if (j < n) cf[j] = (float)c[j];
     }
+    if (tid < 32) R.gmax[tid] = INT_MIN;
     if (tid == 0) {
-        S.status = kRunning; S.it = 0; S.q = -1; S.r = -1; S.tcount = 0;
-        S.degen_run = 0; S.bland = 0; S.flags = 0; S.err = 0; S.z = 0.0; S.dq = 0.0; S.theta = 0.0;
+        R.lcount = 0;
+        S.status = kRunning; S.it = 0; S.degen_run = 0; S.bland = 0; S.flags = 0; S.err = 0; S.k = 0; S.z = 0.0;
     }
     __syncthreads();
 
     for (;;) {
-        if (S.it >= P.max_iters) {
+        const int it = S.it, k = S.k;
+        if (it >= P.max_iters) {
             if (tid == 0) S.status = kIterLimit;
             __syncthreads();
             break;
         }
-        const int it = S.it;
         const bool bland = S.bland != 0;
+        int q = -1;
+        double dq = 0.0;
         // ---- Step 3/4: PRICE + CHUZC
-        bool have_q = false;
         if (P.price_mode == 1 && !bland && Alp != nullptr) {
             // BF16 screen over nonbasic, non-tabu structural columns
-            // four lanes per column, rows dealt round-robin, two chains each
-            for (int base = 0; base < n; base += T / 4) {
-                const int j = base + (tid >> 2), g = tid & 3;
-                const bool live = j < n && pos[j] < 0 && tabu[j] <= it;
-                float a0 = 0.f, a1 = 0.f;
-                if (live) {
-                    int i = g;
-                    for (; i + 4 < m; i += 8) {
-                        a0 = fmaf(y32[i], bf16f(__ldg(Alp + (size_t)i * n + j)), a0);
-                        a1 = fmaf(y32[i + 4], bf16f(__ldg(Alp + (size_t)(i + 4) * n + j)), a1);
-                    }
-                    for (; i < m; i += 4) a0 = fmaf(y32[i], bf16f(__ldg(Alp + (size_t)i * n + j)), a0);
-                }
-                float acc = a0 + a1;
-                acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-                acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-                if (g == 0 && j < n) dts[j] = live ? (float)c[j] - acc : -FLT_MAX;
+            float acc[VC];
+            bool live[VC];
+#pragma unroll
+            for (int v = 0; v < VC; ++v) {
+                const int j = tid + T * v;
+                live[v] = j < n && pos[j] < 0 && tabu[j] <= it;
+                acc[v] = 0.f;
             }
+#pragma unroll 4
+            for (int t = 0; t < k; ++t) {
+                const float yt = y32[t];
+                const uint16_t* row = Alp + (size_t)srow[t] * n;
+#pragma unroll
+                for (int v = 0; v < VC; ++v)
+                    if (live[v]) acc[v] = fmaf(yt, bf16f(__ldg(row + tid + T * v)), acc[v]);
+            }
+            int key[VC], top = INT_MIN;
+#pragma unroll
+            for (int v = 0; v < VC; ++v) {
+                key[v] = live[v] ? fkey(cf[tid + T * v] - acc[v]) : INT_MIN;
+                top = max(top, key[v]);
+            }
+            if (top != INT_MIN) atomicMax(&R.gmax[lane], top);
             __syncthreads();
+            // The K-th largest of the 32 lanes' maxima is at most the K-th largest
+            // column: the columns at or above it hold the top K (about 10 of them).
             const int K = P.topk < kBatchTopk ? P.topk : kBatchTopk;
-            batch_topk<T>(dts, n, K, cand, R.kj, R.kd);
-            // exact FP64 re-price: one warp per candidate
-            const int warp = tid >> 5, lane = tid & 31;
-            for (int t = warp; t < K; t += T / 32) {
-                const int j = cand[t];
-                if (j < 0) continue;
-                double acc = 0.0;
-                for (int i = lane; i < m; i += 32) acc = fma(y[i], __ldg(A + (size_t)i * n + j), acc);
-                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                if (lane == 0) cand_d[t] = c[j] - acc;
+            const int g = R.gmax[lane];
+            int rank = 0;
+#pragma unroll 8
+            for (int o = 0; o < 32; ++o) {
+                const int x = __shfl_sync(0xffffffffu, g, o);
+                rank += x > g || (x == g && o < lane);
             }
-            // best exact slack (non-tabu)
-            BCand bs = {LLONG_MIN, -1};
-            for (int i = tid; i < m; i += T) {
-                const int j = n + i;
-                const long long kd = dkey(-y[i]);
-                if (pos[j] < 0 && tabu[j] <= it && bc_beats(kd, j, bs.d, bs.j)) bs = {kd, j};
-            }
+            const int tau = max(__shfl_sync(0xffffffffu, g, __ffs(__ballot_sync(0xffffffffu, rank == K - 1)) - 1),
+                                INT_MIN + 1);
+#pragma unroll
+            for (int v = 0; v < VC; ++v)
+                if (key[v] >= tau) {
+                    const int e = atomicAdd(&R.lcount, 1);
+                    if (e < 32) { R.lkey[e] = key[v]; R.lj[e] = tid + T * v; }
+                }
             __syncthreads();
-            bs = block_best<T>(bs, R.bc);
-            if (tid == 0) {
-                BCand best = bs;
-                for (int t = 0; t < K; ++t)
-                    if (cand[t] >= 0 && bc_beats(dkey(cand_d[t]), cand[t], best.d, best.j)) best = {dkey(cand_d[t]), cand[t]};
-                if (best.j >= 0 && best.d > dkey(P.tol_d)) {
-                    S.q = best.j;
-                    S.dq = kdouble(best.d);
-                    R.iv[0] = 1;
-                } else {
-                    R.iv[0] = 0;
+            int cnt = R.lcount;
+            if (cnt <= 32) {
+                // rank the list (larger key, then smaller index); every warp alike
+                const int lk = lane < cnt ? R.lkey[lane] : INT_MIN, lj = lane < cnt ? R.lj[lane] : INT_MAX;
+                int lr = lane;
+                if (cnt > K) {
+                    lr = 0;
+                    for (int o = 0; o < cnt; ++o) {
+                        const int ok = __shfl_sync(0xffffffffu, lk, o), oj = __shfl_sync(0xffffffffu, lj, o);
+                        lr += ok > lk || (ok == lk && oj < lj);
+                    }
+                }
+                if (lane < cnt && lr < K) R.sel[warp][lr] = lj;
+                __syncwarp();
+            } else {
+                // more equal columns than the list holds: K rounds of block argmax
+                bool taken[VC];
+#pragma unroll
+                for (int v = 0; v < VC; ++v) taken[v] = key[v] < tau;
+                for (int x = 0; x < K; ++x) {
+                    long long bk = LLONG_MIN;
+                    int bj = -1;
+#pragma unroll
+                    for (int v = 0; v < VC; ++v)
+                        if (!taken[v] && beats(key[v], tid + T * v, bk, bj)) { bk = key[v]; bj = tid + T * v; }
+                    block_best<T>(bk, bj, R, bk, bj);
+#pragma unroll
+                    for (int v = 0; v < VC; ++v) taken[v] |= bj == tid + T * v;
+                    if (lane == 0) R.sel[warp][x] = bj;
+                }
+                __syncwarp();
+                cnt = K;
+            }
+            cnt = min(cnt, K);
+            // exact FP64 re-price: eight lanes per candidate
+            const int id = tid >> 3, g8 = tid & 7;
+            {
+                const bool mine = id < cnt;
+                const int j = mine ? R.sel[warp][id] : 0;
+                double a = 0.0;
+                if (4 * warp < cnt) {
+                    if (mine)
+                        for (int t = g8; t < k; t += 8) a = fma(y[t], __ldg(A + (size_t)srow[t] * n + j), a);
+                    a += __shfl_xor_sync(0xffffffffu, a, 4);
+                    a += __shfl_xor_sync(0xffffffffu, a, 2);
+                    a += __shfl_xor_sync(0xffffffffu, a, 1);
+                    if (mine && g8 == 0) { R.cd[id] = c[j] - a; R.cj[id] = j; }
                 }
             }
             __syncthreads();
-            have_q = R.iv[0] != 0;
-            __syncthreads();
+            // the best of them and of the non-tabu slacks (d = -y), every warp alike
+            long long bk = LLONG_MIN;
+            int bj = -1;
+            if (lane < cnt) { bk = dkey(R.cd[lane]); bj = R.cj[lane]; }
+            for (int t = lane; t < k; t += 32) {
+                const int j = n + srow[t];
+                const long long kd = dkey(-y[t]);
+                if (tabu[j] <= it && beats(kd, j, bk, bj)) { bk = kd; bj = j; }
+            }
+            long long kb;
+            const int win = warp_argmax_key(bk, bj, bj >= 0, kb);
+            if (win >= 0 && kb > ktol) {
+                q = __shfl_sync(0xffffffffu, bj, win);
+                dq = kdouble(kb);
+            }
         }
-        if (!have_q) {
+        if (q < 0) {
             // full FP64 PRICE (the oracle's rule, tabu and aspiration included)
-            BCand ball = {LLONG_MIN, -1}, bnt = {LLONG_MIN, -1};
-            int jmin = -1;
-            const long long ktol = dkey(P.tol_d);
+            double d[VC];
+#pragma unroll
+            for (int v = 0; v < VC; ++v) d[v] = 0.0;
+            for (int t = 0; t < k; ++t) {
+                const double yt = y[t];
+                const double* row = A + (size_t)srow[t] * n;
+#pragma unroll
+                for (int v = 0; v < VC; ++v)
+                    if (tid + T * v < n) d[v] = fma(yt, __ldg(row + tid + T * v), d[v]);
+            }
+            long long ka = LLONG_MIN, kn = LLONG_MIN, km = LLONG_MIN;
+            int ja = -1, jn = -1, jm = -1;
             auto offer = [&](double dv, int j) {
-                const long long d = dkey(dv);
-                if (bc_beats(d, j, ball.d, ball.j)) ball = {d, j};
-                if (tabu[j] <= it && bc_beats(d, j, bnt.d, bnt.j)) bnt = {d, j};
-                if (d > ktol && (jmin < 0 || j < jmin)) jmin = j;
+                const long long kd = dkey(dv);
+                if (beats(kd, j, ka, ja)) { ka = kd; ja = j; }
+                if (tabu[j] <= it && beats(kd, j, kn, jn)) { kn = kd; jn = j; }
+                if (kd > ktol && (jm < 0 || j < jm)) jm = j;
             };
-            // structural columns: four lanes per column
-            for (int base = 0; base < n; base += T / 4) {
-                const int j = base + (tid >> 2), g = tid & 3;
-                const bool live = j < n && pos[j] < 0;
-                double a0 = 0.0, a1 = 0.0;
-                if (live) {
-                    int i = g;
-                    for (; i + 4 < m; i += 8) {
-                        a0 = fma(y[i], __ldg(A + (size_t)i * n + j), a0);
-                        a1 = fma(y[i + 4], __ldg(A + (size_t)(i + 4) * n + j), a1);
-                    }
-                    for (; i < m; i += 4) a0 = fma(y[i], __ldg(A + (size_t)i * n + j), a0);
-                }
-                double acc = a0 + a1;
-                acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-                acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-                if (g == 0 && live) offer(c[j] - acc, j);
+#pragma unroll
+            for (int v = 0; v < VC; ++v) {
+                const int j = tid + T * v;
+                if (j < n) d[v] = c[j] - d[v];
+                if (j < n && pos[j] < 0) offer(d[v], j);
             }
-            for (int i = tid; i < m; i += T)
-                if (pos[n + i] < 0) offer(-y[i], n + i);
-            ball = block_best<T>(ball, R.bc);
-            bnt = block_best<T>(bnt, R.bc);
-            // smallest improving index: reduce as argmax of (-j)
-            BCand bm = {jmin >= 0 ? -(long long)jmin : LLONG_MIN, jmin};
-            bm = block_best<T>(bm, R.bc);
-            if (tid == 0) {
-                if (ball.j < 0 || !(ball.d > ktol)) {
-                    S.status = kOptimal;
-                } else if (bland) {
-                    // d of the smallest improving index: recompute exactly below
-                    S.q = bm.j;
-                    S.flags |= kTfBland;
-                } else if (bnt.j >= 0 && bnt.d > ktol) {
-                    S.q = bnt.j;
-                    S.dq = kdouble(bnt.d);
-                } else {
-                    S.q = ball.j;
-                    S.dq = kdouble(ball.d);
-                    S.flags |= kTfAspiration;
-                }
-            }
-            __syncthreads();
-            if (S.status != kRunning) break;
+            for (int t = tid; t < k; t += T) offer(-y[t], n + srow[t]);
+            block_best<T>(ka, ja, R, ka, ja);
+            block_best<T>(kn, jn, R, kn, jn);
             if (bland) {
-                // exact d of the Bland choice (same arithmetic as above)
-                const int j = S.q;
-                if (tid == 0) {
-                    if (j < n) {
-                        double acc = 0.0;
-                        for (int i = 0; i < m; ++i) acc = fma(y[i], __ldg(A + (size_t)i * n + j), acc);
-                        S.dq = c[j] - acc;
-                    } else {
-                        S.dq = -y[j - n];
-                    }
-                }
+                // smallest improving index: argmax of -j
+                km = jm >= 0 ? -(long long)jm : LLONG_MIN;
+                block_best<T>(km, jm, R, km, jm);
+            }
+            if (ja < 0 || !(ka > ktol)) {
+                if (tid == 0) S.status = kOptimal;
                 __syncthreads();
+                break;
+            }
+            if (bland) {
+                q = jm;
+#pragma unroll
+                for (int v = 0; v < VC; ++v)
+                    if (tid + T * v == q) R.dq = d[v];
+                if (q >= n && tid == 0) R.dq = -y[rslot[q - n]];
+                __syncthreads();
+                dq = R.dq;
+                if (tid == 0) S.flags |= kTfBland;
+            } else if (jn >= 0 && kn > ktol) {
+                q = jn;
+                dq = kdouble(kn);
+            } else {
+                q = ja;
+                dq = kdouble(ka);
+                if (tid == 0) S.flags |= kTfAspiration;
             }
         }
-        const int q = S.q;
         // ---- Step 5: FTRAN alpha = B^-1 a_q
-        for (int k = tid; k < m; k += T) aq[k] = q < n ? __ldg(A + (size_t)k * n + q) : (k == q - n ? 1.0 : 0.0);
-        __syncthreads();
         if (q < n) {
-            // four lanes per row, columns of B^-1 dealt round-robin
-            for (int base = 0; base < m; base += T / 4) {
-                const int i = base + (tid >> 2), g = tid & 3;
-                double a0 = 0.0, a1 = 0.0;
-                if (i < m) {
-                    int k = g;
-                    for (; k + 4 < m; k += 8) {
-                        a0 = fma(Binv[(size_t)k * m + i], aq[k], a0);
-                        a1 = fma(Binv[(size_t)(k + 4) * m + i], aq[k + 4], a1);
-                    }
-                    for (; k < m; k += 4) a0 = fma(Binv[(size_t)k * m + i], aq[k], a0);
-                }
-                double acc = a0 + a1;
-                acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-                acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-                if (g == 0 && i < m) al[i] = acc;
+            for (int i = tid; i < m; i += T) {
+                const double v = __ldg(A + (size_t)i * n + q);
+                if (rslot[i] >= 0) aq[rslot[i]] = v;
+                else au[pos[n + i]] = v;
             }
         } else {
-            for (int i = tid; i < m; i += T) al[i] = Binv[(size_t)(q - n) * m + i];
+            const int unit = rslot[q - n];
+            for (int t = tid; t < k; t += T) aq[t] = t == unit ? 1.0 : 0.0;
         }
         __syncthreads();
-        // ratios one row per lane: a warp-wide division covers 32 rows
-        const long long kpiv = dkey(P.tol_piv);
-        long long tl = dkey(DBL_MAX);
-        for (int i = tid; i < m; i += T) {
-            const double a = al[i];
-            const double t = dkey(a) > kpiv ? bbar[i] / a : DBL_MAX;
-            th[i] = t;
-            tl = min(tl, dkey(t));
+        double al[VR], th[VR];
+        long long kth[VR], kmin = kbig;
+#pragma unroll
+        for (int v = 0; v < VR; ++v) {
+            const int i = tid + T * v;
+            double a0 = 0.0, a1 = 0.0;
+            kth[v] = kbig;
+            al[v] = th[v] = 0.0;
+            if (i < m) {
+                int t = 0;
+#pragma unroll 2
+                for (; t + 1 < k; t += 2) {
+                    a0 = fma(col(t)[i], aq[t], a0);
+                    a1 = fma(col(t + 1)[i], aq[t + 1], a1);
+                }
+                if (t < k) a0 = fma(col(t)[i], aq[t], a0);
+                if (q < n && basis[i] >= n) a1 += au[i];
+                al[v] = a0 + a1;
+                // ratios one row per lane: a warp-wide division covers 32 rows
+                if (dkey(al[v]) > kpiv) {
+                    th[v] = bbar[i] / al[v];
+                    kth[v] = dkey(th[v]);
+                }
+            }
+            kmin = min(kmin, kth[v]);
         }
         // ---- Step 6: CHUZR with the tie set (on integer keys)
-        const long long kmin = block_min_key<T>(tl, R.kv, P.tol_tie, &R.kv[32]);
-        if (kmin == dkey(DBL_MAX)) {
+        kmin = warp_min_key(kmin);
+        if (lane == 0) R.wk[warp] = kmin;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < W; ++w) kmin = min(kmin, R.wk[w]);
+        if (kmin == kbig) {
             if (tid == 0) S.status = kUnbounded;
             __syncthreads();
             break;
         }
-        const long long kthr = R.kv[32];
-        RCand rc = {0, 0, -1};
-        int cnt = 0;
-        for (int i = tid; i < m; i += T) {
-            const long long ka = dkey(al[i]);
-            if (ka > kpiv && dkey(th[i]) <= kthr) {
-                cnt++;
-                RCand x = {ka, basis[i], i};
-                if (rc_beats(x, rc, bland)) rc = x;
+        // (max(1, |t|) by its bits: FP64 compares would cost the pipe as much as the FMA)
+        const double tmin = kdouble(kmin);
+        const long long mag = __double_as_longlong(tmin) & 0x7fffffffffffffffLL;
+        const long long kthr = dkey(tmin + P.tol_tie * __longlong_as_double(max(mag, __double_as_longlong(1.0))));
+        {
+            // the warp's best tied row: largest alpha, exact ties to the smallest basic
+            // variable (Bland: the smallest basic variable)
+            long long ka = LLONG_MIN;
+            int var = INT_MAX, row = -1, cnt = 0;
+            double bt = 0.0, ba = 0.0;
+#pragma unroll
+            for (int v = 0; v < VR; ++v)
+                if (kth[v] <= kthr && kth[v] != kbig) {
+                    const int x = basis[tid + T * v];
+                    const long long kv = dkey(al[v]);
+                    ++cnt;
+                    if (row < 0 || (bland ? x < var : (kv > ka || (kv == ka && x < var)))) {
+                        ka = kv; var = x; row = tid + T * v; bt = th[v]; ba = al[v];
+                    }
+                }
+            const unsigned bal = __ballot_sync(0xffffffffu, row >= 0);
+            int win = bal ? __ffs(bal) - 1 : 0;
+            if (bal && (__popc(bal) > 1 || __any_sync(0xffffffffu, cnt > 1))) {
+                long long kb;
+                win = bland ? warp_argmin_index(var, row >= 0) : warp_argmax_key(ka, var, row >= 0, kb);
+                cnt = __reduce_add_sync(0xffffffffu, cnt);
+            }
+            if (lane == win) { R.wj[warp] = row; R.wv[warp] = var; R.wc[warp] = cnt; R.wa[warp] = ba; R.wt[warp] = bt; }
+        }
+        __syncthreads();
+        int r = -1, leave = 0, ties = 0, bw = 0;
+        {
+            long long ka = LLONG_MIN;
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                if (R.wj[w] < 0) continue;
+                const long long kv = dkey(R.wa[w]);
+                ties += R.wc[w];
+                if (r < 0 || (bland ? R.wv[w] < leave : (kv > ka || (kv == ka && R.wv[w] < leave)))) {
+                    ka = kv; leave = R.wv[w]; r = R.wj[w]; bw = w;
+                }
             }
         }
-        rc = block_row<T>(rc, bland, R.rc, cnt, R.iv);  // best row and tie-set size together
-        const int r = rc.row;
-        const double ar = al[r];
-        const double theta = th[r];
-        const double dq = S.dq;
-        // ---- Step 7/8 bookkeeping (tabu, trace, objective, basis)
-        if (tid == 0) {
+        const double ar = R.wa[bw], theta = R.wt[bw];
+        // ---- Step 7/8: the slots after the pivot, rho and y (in the new slot order)
+        const int join = leave >= n ? leave - n : -1, ent = q >= n ? q - n : -1;
+        const int te = ent >= 0 ? rslot[ent] : -1;
+        const int J = join >= 0 ? (ent >= 0 ? te : k) : -1;             // the joining row's slot
+        const int src = ent >= 0 && join < 0 && te != k - 1 ? k - 1 : -1;  // slot that moves to te
+        const int kn = k + (join >= 0) - (ent >= 0);
+        const int srcrow = src >= 0 ? srow[src] : -1;
+        for (int t = tid; t < kn; t += T) {
+            const int o = t == te && src >= 0 ? src : t;
+            const double rn = (t == J ? 1.0 : col(o)[r]) / ar;
+            const double yo = t == J ? 0.0 : y[o];
+            rho[t] = rn;
+            const double yn = __dadd_rn(yo, __dmul_rn(dq, rn));
+            y[t] = yn;
+            y32[t] = (float)yn;
+        }
+        __syncthreads();
+        // bookkeeping (tabu, trace, objective, basis, slots)
+        if (tid == T - 1) {
             int flags = S.flags;
-            const int leave = basis[r];
             const bool degenerate = theta <= P.tol_tie;
             if (degenerate) flags |= kTfDegenerate;
-            if (P.tabu_tenure > 0 && (cnt > 1 || degenerate)) {
+            if (P.tabu_tenure > 0 && (ties > 1 || degenerate)) {
                 tabu[leave] = it + 1 + P.tabu_tenure;
                 flags |= kTfTabuPush;
             }
-            if (cnt > 1) flags |= kTfTieSet;
+            if (ties > 1) flags |= kTfTieSet;
             if (s.trace_q && it < P.trace_cap) {
                 s.trace_q[(size_t)lp * P.trace_cap + it] = q;
                 s.trace_r[(size_t)lp * P.trace_cap + it] = r;
             }
             S.z = __dadd_rn(S.z, __dmul_rn(dq, theta));
             pos[leave] = -1;
-            basis[r] = q;
-            pos[q] = r;
+            basis[r] = (int16_t)q;
+            pos[q] = (int16_t)r;
+            if (ent >= 0) rslot[ent] = -1;
+            if (src >= 0) { srow[te] = (int16_t)srcrow; rslot[srcrow] = (int16_t)te; }
+            if (join >= 0) { srow[J] = (int16_t)join; rslot[join] = (int16_t)J; }
+            S.k = kn;
             S.it = it + 1;
             S.degen_run = degenerate ? S.degen_run + 1 : 0;
             if (S.bland && !degenerate) S.bland = 0;
             if (!S.bland && P.bland_after > 0 && S.degen_run >= P.bland_after) S.bland = 1;
             S.flags = 0;
+            R.lcount = 0;
         }
-        // ---- Step 8: tableau pivot (row r / alpha_r, row i - alpha_i * row r)
-        for (int k = tid; k < m; k += T) rho[k] = Binv[(size_t)k * m + r] / ar;
-        __syncthreads();
-        for (int k = tid; k < m; k += T) {
-            y[k] = __dadd_rn(y[k], __dmul_rn(dq, rho[k]));
-            y32[k] = (float)y[k];
-        }
-        for (int i = tid; i < m; i += T)
-            bbar[i] = (i == r) ? theta : __dsub_rn(bbar[i], __dmul_rn(al[i], theta));
-        {
-            // element e = k*m + i walks by T: advance (k, i) without dividing
-            const int dk = T / m, di = T - dk * m;
-            int k = tid / m, i = tid - k * m;
-            for (int e = tid; e < m * m; e += T) {
-                Binv[e] = (i == r) ? rho[k] : fma(-al[i], rho[k], Binv[e]);
-                k += dk;
-                i += di;
-                if (i >= m) { i -= m; ++k; }
+        if (tid < 32) R.gmax[tid] = INT_MIN;
+        // ---- Step 8: own rows of bbar and of the live columns
+#pragma unroll
+        for (int v = 0; v < VR; ++v) {
+            const int i = tid + T * v;
+            if (i >= m) continue;
+            const double na = -al[v];
+            bbar[i] = i == r ? theta : __dsub_rn(bbar[i], __dmul_rn(al[v], theta));
+#pragma unroll 4
+            for (int t = 0; t < kn; ++t) {
+                const double old = t == J ? 0.0 : col(t == te && src >= 0 ? src : t)[i];
+                col(t)[i] = i == r ? rho[t] : fma(na, rho[t], old);
             }
         }
         __syncthreads();
         // ---- periodic reinversion (structure-aware, as in the single-LP solver)
-        if (P.reinvert_every > 0 && S.it % P.reinvert_every == 0) {
+        if (P.reinvert_every > 0 && (it + 1) % P.reinvert_every == 0) {
             if (tid == 0) {
-                int k = 0, kr = 0;
+                int kp = 0, kr = 0;
                 for (int p = 0; p < m; ++p)
-                    if (basis[p] < n) lstP[k++] = p;
+                    if (basis[p] < n) lstP[kp++] = (int16_t)p;
                 for (int i = 0; i < m; ++i)
-                    if (pos[n + i] < 0) lstR[kr++] = i;
-                S.k = k;
-                if (k != kr) S.err = 1;
+                    if (rslot[i] >= 0) lstR[kr++] = (int16_t)i;
+                if (kp != kn || kr != kn) S.err = 1;
             }
             __syncthreads();
-            const int k = S.k;
+            const int kk = kn;
             if (S.err) { if (tid == 0) S.status = -1; __syncthreads(); break; }
-            for (int e = tid; e < k * k; e += T) {
-                const int t = e / k, a = e - t * k;
-                W[e] = __ldg(A + (size_t)lstR[a] * n + basis[lstP[t]]);
+            for (int e = tid; e < kk * kk; e += T) {
+                const int t = e / kk, a = e - t * kk;
+                Wm[e] = __ldg(A + (size_t)lstR[a] * n + basis[lstP[t]]);
             }
-            for (int a = tid; a < k; a += T) { pinv[a] = 0; pivrow[a] = -1; }  // pinv doubles as "row used"
+            for (int a = tid; a < kk; a += T) { pinv[a] = 0; pivrow[a] = -1; }  // pinv doubles as "row used"
             __syncthreads();
-            for (int j = 0; j < k; ++j) {
-                BCand pc = {LLONG_MIN, -1};
-                for (int a = tid; a < k; a += T)
+            for (int j = 0; j < kk; ++j) {
+                long long pk = LLONG_MIN;
+                int p = -1;
+                for (int a = tid; a < kk; a += T)
                     if (!pinv[a]) {
-                        const long long v = dkey(fabs(W[(size_t)j * k + a]));
-                        if (bc_beats(v, a, pc.d, pc.j)) pc = {v, a};
+                        const long long v = dkey(fabs(Wm[(size_t)j * kk + a]));
+                        if (beats(v, a, pk, p)) { pk = v; p = a; }
                     }
-                pc = block_best<T>(pc, R.bc);
-                if (pc.j < 0 || !(pc.d > 0)) {
+                block_best<T>(pk, p, R, pk, p);
+                if (p < 0 || !(pk > 0)) {
                     if (tid == 0) S.err = 2;
                     __syncthreads();
                     break;
                 }
-                const int p = pc.j;
-                for (int a = tid; a < k; a += T) rho[a] = W[(size_t)j * k + a];  // pivot column f
+                for (int a = tid; a < kk; a += T) rho[a] = Wm[(size_t)j * kk + a];  // pivot column f
                 __syncthreads();
                 const double pv = rho[p];
-                for (int t = tid; t < k; t += T) aq[t] = W[(size_t)t * k + p] / pv;  // g_t (row p / pivot)
-                if (tid == 0) { pivrow[j] = p; pinv[p] = 1; }
+                for (int t = tid; t < kk; t += T) aq[t] = Wm[(size_t)t * kk + p] / pv;  // g_t (row p / pivot)
+                if (tid == 0) { pivrow[j] = (int16_t)p; pinv[p] = 1; }
                 __syncthreads();
-                for (int e = tid; e < k * k; e += T) {
-                    const int t = e / k, a = e - t * k;
-                    if (t == j) W[e] = (a == p) ? 1.0 / pv : -rho[a] / pv;
-                    else W[e] = (a == p) ? aq[t] : fma(-rho[a], aq[t], W[e]);
+                for (int e = tid; e < kk * kk; e += T) {
+                    const int t = e / kk, a = e - t * kk;
+                    if (t == j) Wm[e] = (a == p) ? 1.0 / pv : -rho[a] / pv;
+                    else Wm[e] = (a == p) ? aq[t] : fma(-rho[a], aq[t], Wm[e]);
                 }
                 __syncthreads();
             }
             if (S.err) { if (tid == 0) S.status = -1; __syncthreads(); break; }
-            for (int t = tid; t < k; t += T) pinv[pivrow[t]] = t;
-            for (int e = tid; e < m * m; e += T) Binv[e] = 0.0;
-            __syncthreads();
-            // B11^-1[bb][a] = W[pinv[a]*k + pivrow[bb]]
-            for (int e = tid; e < k * k; e += T) {
-                const int bb = e / k, a = e - bb * k;
-                Binv[(size_t)lstR[a] * m + lstP[bb]] = W[(size_t)pinv[a] * k + pivrow[bb]];
+            for (int t = tid; t < kk; t += T) {
+                pinv[pivrow[t]] = (int16_t)t;
+                srow[t] = lstR[t];
+                rslot[lstR[t]] = (int16_t)t;
             }
-            // slack positions: B^-1[p, s] = 1, B^-1[p, R[a]] = -sum_b A[s, J[b]] B11^-1[b][a]
-            for (int e = tid; e < m * k; e += T) {
-                const int p = e / (k > 0 ? k : 1), a = e - p * k;
-                if (k == 0 || basis[p] < n) continue;
+            __syncthreads();
+            // B11^-1[bb][a] = Wm[pinv[a]*kk + pivrow[bb]]
+            for (int e = tid; e < kk * kk; e += T) {
+                const int bb = e / kk, a = e - bb * kk;
+                col(a)[lstP[bb]] = Wm[(size_t)pinv[a] * kk + pivrow[bb]];
+            }
+            // slack positions: B^-1[p, R[a]] = -sum_b A[s, J[b]] B11^-1[b][a]
+            for (int e = tid; e < m * kk; e += T) {
+                const int p = e / (kk > 0 ? kk : 1), a = e - p * kk;
+                if (kk == 0 || basis[p] < n) continue;
                 const int sr = basis[p] - n;
                 double acc = 0.0;
-                for (int bb = 0; bb < k; ++bb)
-                    acc = fma(__ldg(A + (size_t)sr * n + basis[lstP[bb]]), W[(size_t)pinv[a] * k + pivrow[bb]], acc);
-                Binv[(size_t)lstR[a] * m + p] = -acc;
+                for (int bb = 0; bb < kk; ++bb)
+                    acc = fma(__ldg(A + (size_t)sr * n + basis[lstP[bb]]), Wm[(size_t)pinv[a] * kk + pivrow[bb]], acc);
+                col(a)[p] = -acc;
             }
-            for (int p = tid; p < m; p += T)
-                if (basis[p] >= n) Binv[(size_t)(basis[p] - n) * m + p] = 1.0;
             __syncthreads();
             for (int p = tid; p < m; p += T) {
-                double acc = 0.0;
-                for (int kk = 0; kk < m; ++kk) acc = fma(Binv[(size_t)kk * m + p], b[kk], acc);
+                double acc = basis[p] >= n ? b[basis[p] - n] : 0.0;
+                for (int t = 0; t < kk; ++t) acc = fma(col(t)[p], b[srow[t]], acc);
                 bbar[p] = acc;
             }
-            for (int sr = tid; sr < m; sr += T) {
+            for (int t = tid; t < kk; t += T) {
                 double acc = 0.0;
-                for (int p = 0; p < m; ++p)
-                    if (basis[p] < n) acc = fma(c[basis[p]], Binv[(size_t)sr * m + p], acc);
-                y[sr] = acc;
-                y32[sr] = (float)acc;
+                for (int bb = 0; bb < kk; ++bb) acc = fma(c[basis[lstP[bb]]], col(t)[lstP[bb]], acc);
+                y[t] = acc;
+                y32[t] = (float)acc;
             }
             __syncthreads();
-            double zz = 0.0;
-            for (int p = tid; p < m; p += T)
-                if (basis[p] < n) zz = fma(c[basis[p]], bbar[p], zz);
-            zz = block_sum<T>(zz, R.dv);
-            if (tid == 0) S.z = zz;
+            if (warp == 0) {
+                double zz = 0.0;
+                for (int bb = lane; bb < kk; bb += 32) zz = fma(c[basis[lstP[bb]]], bbar[lstP[bb]], zz);
+                zz = warp_sum(zz);
+                if (lane == 0) S.z = zz;
+            }
             __syncthreads();
         }
     }
     // ---- outputs
     double* xo = s.x + L.c_off;
     double* yo = s.y + L.r_off;
-    for (int j = tid; j < n; j += T) xo[j] = 0.0;
-    __syncthreads();
-    for (int p = tid; p < m; p += T)
-        if (basis[p] < n) xo[basis[p]] = bbar[p];
-    for (int i = tid; i < m; i += T) yo[i] = y[i];
+    for (int j = tid; j < n; j += T) xo[j] = pos[j] >= 0 ? bbar[pos[j]] : 0.0;
+    for (int i = tid; i < m; i += T) yo[i] = rslot[i] >= 0 ? y[rslot[i]] : 0.0;
     if (tid == 0) {
         s.status[lp] = S.status;
         s.iters[lp] = S.it;
@@ -680,8 +632,9 @@ __device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, doub
     __syncthreads();
 }
 
-template <int T, bool SMEM>
-__global__ void __launch_bounds__(T, 1024 / T) k_batch(BatchState s, int bucket, int begin, int count, int mmax, int nmax) {
+template <int T>
+__global__ void __launch_bounds__(T, 1024 / T) k_batch(BatchState s, int bucket, int begin, int count, int mmax, int nmax,
+                                                       int ks) {
     extern __shared__ __align__(16) unsigned char smem[];
     double* slot = s.scratch[bucket] + (size_t)blockIdx.x * s.slot_doubles[bucket];
     __shared__ int next;
@@ -691,26 +644,28 @@ __global__ void __launch_bounds__(T, 1024 / T) k_batch(BatchState s, int bucket,
         const int k = next;
         __syncthreads();
         if (k >= count) break;
-        solve_one<T, SMEM>(s, s.order[begin + k], smem, slot, mmax, nmax);
+        solve_one<T>(s, s.order[begin + k], smem, slot, mmax, nmax, ks);
     }
 }
 
 }  // namespace
 
-size_t batch_smem_bytes(int mmax, int nmax, bool smem_binv) {
-    size_t d = (smem_binv ? (size_t)mmax * mmax : 0) + 6 * (size_t)mmax;
-    size_t f = (size_t)mmax + nmax;
-    size_t i = 3 * (size_t)mmax + 2 * ((size_t)nmax + mmax) + 2 * (size_t)mmax + kBatchTopk + 1;
-    return d * 8 + f * 4 + i * 4 + 8 + (kBatchTopk + 1) * 8 + 64;
+// ks live columns in shared memory beside the vectors
+size_t batch_smem_bytes(int mmax, int nmax, int ks) {
+    const size_t d = (size_t)ks * mmax + 5 * (size_t)mmax;
+    const size_t f = (size_t)mmax + nmax;
+    const size_t i = (size_t)nmax + mmax;
+    const size_t h = 7 * (size_t)mmax + nmax + mmax;
+    return d * 8 + f * 4 + i * 4 + h * 2;
 }
 
-using BatchKernel = void (*)(BatchState, int, int, int, int, int);
+using BatchKernel = void (*)(BatchState, int, int, int, int, int, int);
 
-BatchKernel batch_kernel(int threads, bool smem_binv) {
+BatchKernel batch_kernel(int threads) {
     switch (threads) {
-        case 128: return smem_binv ? k_batch<128, true> : k_batch<128, false>;
-        case 256: return smem_binv ? k_batch<256, true> : k_batch<256, false>;
-        default: return smem_binv ? k_batch<512, true> : k_batch<512, false>;
+        case 128: return k_batch<128>;
+        case 256: return k_batch<256>;
+        default: return k_batch<512>;
     }
 }
 
@@ -731,8 +686,11 @@ struct lp_batch {
     std::vector<BatchLP> lps;
     std::vector<int32_t> order;
     int bucket_begin[kBuckets + 1] = {};
-    int cfg_threads[kBuckets] = {256, 256, 256, 256};
-    int cfg_smem[kBuckets] = {1, 1, 0, 0};
+    int bucket_m[kBuckets] = {}, bucket_n[kBuckets] = {};  // the largest m and n in each bucket
+    // 4096 LPs of m 16..256: 3.31 ms (3.35 with 256 threads throughout, 4.05 with 128, 5.2
+    // with 512; shared-memory columns 3.43); m 16..64 alone 0.44 ms (0.65 with 256)
+    int cfg_threads[kBuckets] = {128, 128, 256, 256};
+    int cfg_smem[kBuckets] = {0, 0, 0, 0};
     int64_t sum_m = 0, sum_n = 0;
     BatchState st{};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -781,16 +739,19 @@ void bfree(lp_batch* h) {
 
 bool cfg_valid(const lp_batch* h, int bucket, int threads, int smem) {
     if (threads != 128 && threads != 256 && threads != 512) return false;
-    const size_t need = batch_smem_bytes(kBucketM[bucket], kBatchMaxN, smem != 0);
+    // (the flag stays tied to sizes whose whole inverse would fit)
+    const size_t need = batch_smem_bytes(kBucketM[bucket], kBatchMaxN, smem ? kBucketM[bucket] : 0);
     return need <= h->smem_optin;
 }
 
 int grid_for(const lp_batch* h, int bucket, int* grid, size_t* smem) {
     const int T = h->cfg_threads[bucket];
     const bool sm = h->cfg_smem[bucket] != 0;
-    *smem = batch_smem_bytes(kBucketM[bucket], kBatchMaxN, sm);
-    BatchKernel k = batch_kernel(T, sm);
-    BCK(cudaFuncSetAttribute(reinterpret_cast<const void*>(k), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem));
+    *smem = batch_smem_bytes(h->bucket_m[bucket], h->bucket_n[bucket], sm ? kSmemCols : 0);
+    BatchKernel k = batch_kernel(T);
+    // (one limit for every bucket: buckets with the same thread count share a kernel)
+    BCK(cudaFuncSetAttribute(reinterpret_cast<const void*>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)batch_smem_bytes(kBatchMaxM, kBatchMaxN, kSmemCols)));
     int occ = 0;
     BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, T, *smem));
     *grid = h->sms * std::max(1, occ);
@@ -830,8 +791,9 @@ int launch_buckets(lp_batch* h, int b0, int b1, const BucketLaunch* plan, bool c
             st = h->bstream[bk];
             BCK(cudaStreamWaitEvent(st, h->fork, 0));
         }
-        BatchKernel k = batch_kernel(h->cfg_threads[bk], h->cfg_smem[bk] != 0);
-        k<<<plan[bk].grid, h->cfg_threads[bk], plan[bk].smem, st>>>(h->st, bk, begin, cnt, kBucketM[bk], kBatchMaxN);
+        BatchKernel k = batch_kernel(h->cfg_threads[bk]);
+        k<<<plan[bk].grid, h->cfg_threads[bk], plan[bk].smem, st>>>(h->st, bk, begin, cnt, h->bucket_m[bk], h->bucket_n[bk],
+                                                                    h->cfg_smem[bk] ? kSmemCols : 0);
         BCK(cudaGetLastError());
         if (concurrent) {
             BCK(cudaEventRecord(h->join[bk], st));
@@ -950,7 +912,11 @@ int lp_batch_create(lp_batch** out, int32_t count, const int32_t* m, const int32
         int k = 0;
         for (int bk = 0; bk < kBuckets; ++bk) {
             h->bucket_begin[bk] = k;
-            while (k < count && bucket_of(idx[k]) == bk) ++k;
+            while (k < count && bucket_of(idx[k]) == bk) {
+                h->bucket_m[bk] = std::max(h->bucket_m[bk], h->lps[idx[k]].m);
+                h->bucket_n[bk] = std::max(h->bucket_n[bk], h->lps[idx[k]].n);
+                ++k;
+            }
         }
         h->bucket_begin[kBuckets] = count;
     }
