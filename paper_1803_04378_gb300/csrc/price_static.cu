@@ -83,6 +83,14 @@ __device__ void block_best(double& d, int& j) {
     }
 }
 
+// At the duals of a solve under way y_i is zero on every row with a basic slack, so
+// only the rows with a nonzero y_i are read when they are few.  The dense pass is
+// bound by the FP64 pipe (an FMA per 8 bytes): 82 us a call at 4096 x 8192.  With one
+// row in twelve the list takes a twelfth of the FMAs and, in 128-byte pieces, 202 of
+// A's 268 MB: 52 us, bound by DRAM.  One row in four: 69 us; one in three would read
+// nearly every piece and gains nothing (dense again).
+constexpr int kSparse = 4;
+
 // d_j = c_j - y^T a_j for nonbasic j (d_{n+i} = -y_i for slacks); the block
 // that finishes last writes the largest d_j > tol_d (exact ties to the
 // smallest j) to q_out / dq_out, or q_out = -1 when none exceeds tol_d.
@@ -102,7 +110,59 @@ __global__ void __launch_bounds__(kThreads) k_price_static(int m, int n, const d
     int best_j = -1;
     const int G = gridDim.x;
     const int owned = (n - (int)blockIdx.x + G - 1) / G;
-    for (int l = warp; l < owned; l += nw) {
+    // The rows with a dual, in increasing order, when they are at most a quarter of
+    // all: each warp counts and then writes those of its run of rows.
+    const int cap = m / kSparse;
+    double* nzv = ysh + me;
+    int* nzi = reinterpret_cast<int*>(nzv + cap);
+    __shared__ int wn[kThreads / 32];
+    const int run = ((m + nw - 1) / nw + 31) & ~31;
+    const int r0 = min(m, warp * run), r1 = min(m, r0 + run);
+    int mine = 0;
+    for (int k = r0; k < r1; k += 32) mine += __popc(__ballot_sync(0xffffffffu, k + lane < r1 && ysh[k + lane] != 0.0));
+    if (lane == 0) wn[warp] = mine;
+    __syncthreads();
+    int nz = 0, at = 0;
+    for (int w = 0; w < nw; ++w) {
+        if (w == warp) at = nz;
+        nz += wn[w];
+    }
+    const bool sparse = nz <= cap;
+    if (sparse) {
+        for (int k = r0; k < r1; k += 32) {
+            const double v = k + lane < r1 ? ysh[k + lane] : 0.0;
+            const unsigned bal = __ballot_sync(0xffffffffu, v != 0.0);
+            if (v != 0.0) {
+                const int e = at + __popc(bal & ((1u << lane) - 1u));
+                nzv[e] = v;
+                nzi[e] = k + lane;
+            }
+            at += __popc(bal);
+        }
+        __syncthreads();
+        // two columns per warp at a time, eight gathers in flight per lane
+        for (int l = warp; l < owned; l += 2 * nw) {
+            const int j0 = blockIdx.x + G * l, j1 = j0 + G * nw;
+            const bool in0 = pos[j0] < 0, in1 = l + nw < owned && pos[j1] < 0;
+            const double* c0 = A + (size_t)j0 * lda;
+            const double* c1 = A + (size_t)(in1 ? j1 : j0) * lda;
+            double a0 = 0.0, a1 = 0.0;
+#pragma unroll 4
+            for (int t = lane; t < nz; t += 32) {
+                const int i = nzi[t];
+                const double v = nzv[t], u0 = __ldg(c0 + i), u1 = __ldg(c1 + i);
+                a0 = fma(u0, v, a0);
+                a1 = fma(u1, v, a1);
+            }
+            const double d0 = c[j0] - warp_sum(a0);
+            if (in0 && better(d0, j0, best_d, best_j)) { best_d = d0; best_j = j0; }
+            if (in1) {  // (uniform over the warp)
+                const double d1 = c[j1] - warp_sum(a1);
+                if (better(d1, j1, best_d, best_j)) { best_d = d1; best_j = j1; }
+            }
+        }
+    }
+    for (int l = warp; l < owned && !sparse; l += nw) {
         const int j = blockIdx.x + G * l;
         if (pos[j] >= 0) continue;
         const double* colp = A + (size_t)j * lda;
@@ -149,6 +209,11 @@ __global__ void __launch_bounds__(kThreads) k_price_static(int m, int n, const d
     }
 }
 
+// y, and the list of its nonzeros
+size_t price_smem(int m) {
+    return (size_t)((m + 1) & ~1) * sizeof(double) + (size_t)(m / kSparse) * (sizeof(double) + sizeof(int));
+}
+
 // Identity of the calling thread's current context (driver entry points
 // looked up through the runtime, so the library needs no libcuda at link
 // time).  Host-only queries: they enqueue nothing and allocate nothing.
@@ -187,7 +252,7 @@ int setup_device(int dev, DeviceSetup** out) {
         void* ptr = nullptr;
         if (cudaGetSymbolAddress(&ptr, g_price_scratch) != cudaSuccess || ptr == nullptr) return LP_ERR_CUDA;
         if (cudaFuncSetAttribute(k_price_static, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(LP_PRICE_STATIC_MAX_M * sizeof(double))) != cudaSuccess)
+                                 (int)price_smem(LP_PRICE_STATIC_MAX_M)) != cudaSuccess)
             return LP_ERR_CUDA;
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
@@ -221,7 +286,7 @@ extern "C" int lp_price_static(int32_t m, int32_t n, const double* A_colmajor, i
     if (blocks > kMaxBlocks) blocks = kMaxBlocks;
     if (blocks > n) blocks = n;
     if (cudaMemsetAsync(&s->scratch->ticket, 0, sizeof(int32_t), st) != cudaSuccess) return LP_ERR_CUDA;
-    const size_t smem = (size_t)((m + 1) & ~1) * sizeof(double);
+    const size_t smem = price_smem(m);
     k_price_static<<<blocks, kThreads, smem, st>>>(m, n, A_colmajor, lda, c, y, pos, tol_d, q_out, dq_out,
                                                    s->scratch);
     if (cudaGetLastError() != cudaSuccess) return LP_ERR_CUDA;
