@@ -17,8 +17,19 @@
 // pass).  FP16 rows are padded to a multiple of 8 elements (16-byte TMA
 // strides); FP32 results keep the logical widths.  Parameters are packed
 // W1, b1, W2, b2, W3, b3 with W_l row-major [in_l x out_l].
+//
+// The element-wise work rides in the GEMMs' epilogues: a lane of an epilogue
+// warp holds 32 columns of one row, so the row-major copy leaves in 16-byte
+// stores and the transposed copy in 64-byte rows of a warp.  (As kernels of
+// their own, with the transposed copy written element by element, they took
+// 220 of a training step's 324 us at batch 256 and 6144 -> 512 -> 512 -> 3072.)
+// Every sum keeps its order -- K by K in the MMA, row by row in the bias
+// gradients -- whatever the tile width, so the results do not depend on it:
+// products with few tiles take 32 columns per CTA (z1 at batch 256: 8 CTAs of 128
+// columns 32 us).  The chain is programmatic dependent launches.
 #include "../../include/lpgb.h"
 #include "lpgb_internal.cuh"
+#include "tc_gemm.cuh"
 
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -29,108 +40,262 @@
 #include <new>
 #include <vector>
 
-namespace lpgb {
-cudaError_t tc_gemm(const void* A, int lda, const void* B, int ldb, float* D, int ldd, int M, int N, int K, bool bf16,
-                    int32_t* err, cudaStream_t st);
-}
+using lpgb::launch_k;
+using lpgb::pdl_enter;
 
 namespace {
 
 inline int pad8(int v) { return (v + 7) & ~7; }
 
-// X (rows x cols, FP32) -> x16 (row stride ld) and xT (cols x rows, row stride ldt), FP16
-__global__ void k_input16(const float* __restrict__ X, int rows, int cols, __half* __restrict__ x16, int ld,
-                          __half* __restrict__ xT, int ldt) {
-    const size_t n = (size_t)rows * cols;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e / cols), c = (int)(e % cols);
-        const __half h = __float2half_rn(X[e]);
-        x16[(size_t)r * ld + c] = h;
-        xT[(size_t)c * ldt + r] = h;
+// 32 consecutive halves of row `row` from column c0 (row stride ld, a multiple
+// of 8, base 16-byte aligned): 16-byte stores where all columns exist
+__device__ __forceinline__ void store_row16(__half* a, int ld, int row, int c0, int N, const __half (&h)[32]) {
+    __half* p = a + (size_t)row * ld + c0;
+    if (c0 + 32 <= N) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 8) *reinterpret_cast<uint4*>(p + i) = *reinterpret_cast<const uint4*>(&h[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (c0 + i < N) p[i] = h[i];
+    }
+}
+// the same as column `row` of the transposed copy: a warp's rows side by side
+__device__ __forceinline__ void store_col16(__half* aT, int ldt, int row, int c0, int N, const __half (&h)[32]) {
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+        if (c0 + i < N) aT[(size_t)(c0 + i) * ldt + row] = h[i];
+}
+__device__ __forceinline__ void load_row32(const float* z, int ld, int row, int c0, int N, float (&v)[32]) {
+    const float* p = z + (size_t)row * ld + c0;
+    if (c0 + 32 <= N && (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(z) & 15) == 0) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(p + i);
+            v[i] = q.x; v[i + 1] = q.y; v[i + 2] = q.z; v[i + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = c0 + i < N ? p[i] : 0.f;
+    }
+}
+__device__ __forceinline__ void store_row32(float* z, int ld, int row, int c0, int N, const float (&v)[32]) {
+    float* p = z + (size_t)row * ld + c0;
+    if (c0 + 32 <= N && (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(z) & 15) == 0) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4*>(p + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (c0 + i < N) p[i] = v[i];
     }
 }
 
-// z += bias (per column); a = relu(z) (relu = 0: a = z) in FP16, row-major
-// (row stride lda) and transposed (row stride ldt)
-__global__ void k_bias_act(float* __restrict__ z, const float* __restrict__ bias, int rows, int cols, int relu,
-                           __half* __restrict__ a, int lda, __half* __restrict__ aT, int ldt) {
-    const size_t n = (size_t)rows * cols;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e / cols), c = (int)(e % cols);
-        const float v = z[e] + bias[c];
-        z[e] = v;
+// D = acc (the weight gradients)
+struct EpiStore {
+    float* D;
+    int M, N;
+    __device__ void operator()(int trow, int m0, int n0, int c0, const float (&v)[32]) const {
+        if (m0 + trow < M) store_row32(D, N, m0 + trow, n0 + c0, N, v);
+    }
+};
+
+// z = acc + bias; with a: a = relu(z) in FP16, and with aT its transpose; z itself where it is asked for
+struct EpiAct {
+    const float* bias;
+    float* z;
+    __half *a, *aT;
+    int lda, ldt, M, N;
+    __device__ void operator()(int trow, int m0, int n0, int c0, const float (&v)[32]) const {
+        const int row = m0 + trow, c = n0 + c0;
+        if (row >= M) return;
+        float x[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) x[i] = v[i] + (c + i < N ? __ldg(bias + c + i) : 0.f);
+        if (z) store_row32(z, N, row, c, N, x);
         if (a) {
-            const __half h = __float2half_rn(relu ? fmaxf(v, 0.f) : v);
-            a[(size_t)r * lda + c] = h;
-            aT[(size_t)c * ldt + r] = h;
+            __align__(16) __half h[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) h[i] = __float2half_rn(fmaxf(x[i], 0.f));
+            store_row16(a, lda, row, c, N, h);
+            if (aT) store_col16(aT, ldt, row, c, N, h);
         }
     }
-}
+};
 
-// dz = (sigmoid(z) - t) / B in FP16 (row-major and transposed); loss partial sums (softplus(z) - t z) / B
-__global__ void k_bce(const float* __restrict__ z, const float* __restrict__ t, int rows, int cols,
-                      __half* __restrict__ dz, int ld, __half* __restrict__ dzT, int ldt, float* __restrict__ loss) {
-    const size_t n = (size_t)rows * cols;
-    const float inv = 1.f / (float)rows;
-    float l = 0.f;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e / cols), c = (int)(e % cols);
-        const float v = z[e], tt = t[e];
-        const float sp = v > 0.f ? v + log1pf(expf(-v)) : log1pf(expf(v));
-        l += (sp - tt * v) * inv;
-        const float sg = 1.f / (1.f + expf(-v));
-        const __half h = __float2half_rn((sg - tt) * inv);
-        dz[(size_t)r * ld + c] = h;
-        dzT[(size_t)c * ldt + r] = h;
+// z = acc + bias; dz = (sigmoid(z) - t) / B in FP16, row-major and transposed; the loss's partial sums
+// (softplus(z) - t z) / B
+struct EpiBce {
+    const float *bias, *t;
+    __half *dz, *dzT;
+    float* loss;
+    int ld, ldt, M, N;
+    __device__ void operator()(int trow, int m0, int n0, int c0, const float (&v)[32]) const {
+        const int row = m0 + trow, c = n0 + c0;
+        const float inv = 1.f / (float)M;
+        float l = 0.f;
+        if (row < M) {
+            float tt[32];
+            load_row32(t, N, row, c, N, tt);
+            __align__(16) __half h[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                if (c + i < N) {
+                    const float x = v[i] + __ldg(bias + c + i);
+                    const float sp = x > 0.f ? x + log1pf(expf(-x)) : log1pf(expf(x));
+                    l += (sp - tt[i] * x) * inv;
+                    const float sg = 1.f / (1.f + expf(-x));
+                    h[i] = __float2half_rn((sg - tt[i]) * inv);
+                } else {
+                    h[i] = __float2half_rn(0.f);
+                }
+            }
+            store_row16(dz, ld, row, c, N, h);
+            store_col16(dzT, ldt, row, c, N, h);
+        }
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
     }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
-}
+};
 
-// dz = da * (z > 0), FP16 (row-major and transposed)
-__global__ void k_relu_back(const float* __restrict__ da, const float* __restrict__ z, int rows, int cols,
-                            __half* __restrict__ dz, int ld, __half* __restrict__ dzT, int ldt) {
-    const size_t n = (size_t)rows * cols;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e / cols), c = (int)(e % cols);
-        const __half h = __float2half_rn(z[e] > 0.f ? da[e] : 0.f);
-        dz[(size_t)r * ld + c] = h;
-        dzT[(size_t)c * ldt + r] = h;
+// dz = acc * (z > 0), FP16 (row-major and transposed)
+struct EpiReluBack {
+    const float* z;
+    __half *dz, *dzT;
+    int ld, ldt, M, N;
+    __device__ void operator()(int trow, int m0, int n0, int c0, const float (&v)[32]) const {
+        const int row = m0 + trow, c = n0 + c0;
+        if (row >= M) return;
+        float zz[32];
+        load_row32(z, N, row, c, N, zz);
+        __align__(16) __half h[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) h[i] = __float2half_rn(zz[i] > 0.f ? v[i] : 0.f);
+        store_row16(dz, ld, row, c, N, h);
+        store_col16(dzT, ldt, row, c, N, h);
+    }
+};
+
+// X (rows x cols, FP32) -> x16 (row stride ld) and, where asked for, xT (cols x
+// rows, row stride ldt), FP16, by 32 x 32 tiles through shared memory; loss = 0
+constexpr int kTile = 32;
+__global__ void __launch_bounds__(256) k_input16(const float* __restrict__ X, int rows, int cols,
+                                                 __half* __restrict__ x16, int ld, __half* __restrict__ xT, int ldt,
+                                                 float* loss) {
+    pdl_enter();
+    __shared__ __half tile[kTile][kTile + 2];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int c0 = blockIdx.x * kTile, r0 = blockIdx.y * kTile;
+    if (loss && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *loss = 0.f;
+#pragma unroll
+    for (int i = 0; i < kTile; i += 8) {
+        const int r = r0 + ty + i, c = c0 + tx;
+        if (r < rows && c < cols) {
+            const __half h = __float2half_rn(X[(size_t)r * cols + c]);
+            x16[(size_t)r * ld + c] = h;
+            tile[ty + i][tx] = h;
+        }
+    }
+    if (!xT) return;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kTile; i += 8) {
+        const int c = c0 + ty + i, r = r0 + tx;
+        if (r < rows && c < cols) xT[(size_t)c * ldt + r] = tile[tx][ty + i];
     }
 }
 
-// db[c] = sum_r dz[r][c] (row stride ld)
-__global__ void k_colsum(const __half* __restrict__ dz, int ld, int rows, int cols, float* __restrict__ db) {
+// db[c] = sum_r dz[r][c], row by row, of the three layers' dz at once (32 rows of
+// loads in flight; one at a time the three sums took 55 us)
+struct ColSum {
+    const __half* dz[3];
+    float* db[3];
+    int ld[3], cols[3];
+};
+__global__ void __launch_bounds__(64) k_colsum(ColSum q, int rows) {
+    pdl_enter();
+    const int l = blockIdx.y;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
+    if (c >= q.cols[l]) return;
+    const __half* p = q.dz[l] + c;
+    const size_t ld = q.ld[l];
     float s = 0.f;
-    for (int r = 0; r < rows; ++r) s += __half2float(dz[(size_t)r * ld + c]);
-    db[c] = s;
-}
-
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m1,
-                       float* __restrict__ m2, size_t n, float lr, float b1, float b2, float eps, float c1,
-                       float c2) {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const float gg = g[e];
-        const float a = b1 * m1[e] + (1.f - b1) * gg;
-        const float v = b2 * m2[e] + (1.f - b2) * gg * gg;
-        m1[e] = a;
-        m2[e] = v;
-        p[e] = p[e] - lr * (a / c1) / (sqrtf(v / c2) + eps);
+    int r = 0;
+    for (; r + 32 <= rows; r += 32) {
+        __half h[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) h[i] = p[(r + i) * ld];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) s += __half2float(h[i]);
     }
+    for (; r < rows; ++r) s += __half2float(p[r * ld]);
+    q.db[l][c] = s;
 }
 
-// FP16 copies of W (rows x cols, FP32 row-major): W itself (row stride ldn)
-// and W^T (cols x rows, row stride ldt)
-__global__ void k_weight16(const float* __restrict__ W, int rows, int cols, __half* __restrict__ Wn, int ldn,
-                           __half* __restrict__ WT, int ldt) {
-    const size_t n = (size_t)rows * cols;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e / cols), c = (int)(e % cols);
-        const __half h = __float2half_rn(W[e]);
-        if (Wn) Wn[(size_t)r * ldn + c] = h;
-        WT[(size_t)c * ldt + r] = h;
+// One Adam step on every parameter (kAdam) and the FP16 copies of the weights from
+// the FP32 masters: W itself (row stride ldn, where asked for) and W^T, by 64 x 32
+// tiles through shared memory.  The blocks past the matrices' tiles take the biases.
+struct Mats {
+    int rows[3], cols[3], tiles_c[3], first[4];  // first tile of each matrix; first[3]: their number
+    size_t off[6];                               // W1 b1 W2 b2 W3 b3
+    int nbias[3];
+    __half *wn[3], *wt[3];
+    int ldn[3], ldt[3];
+};
+struct Adam {
+    float *p, *m1, *m2;
+    const float* g;
+    float lr, b1, b2, eps, c1, c2;
+};
+template <bool kAdam>
+__device__ __forceinline__ float adam_one(const Adam& q, size_t e) {
+    if (!kAdam) return q.p[e];
+    const float gg = q.g[e];
+    const float a = q.b1 * q.m1[e] + (1.f - q.b1) * gg;
+    const float v = q.b2 * q.m2[e] + (1.f - q.b2) * gg * gg;
+    q.m1[e] = a;
+    q.m2[e] = v;
+    const float w = q.p[e] - q.lr * (a / q.c1) / (sqrtf(v / q.c2) + q.eps);
+    q.p[e] = w;
+    return w;
+}
+constexpr int kWR = 64, kWC = 32;
+template <bool kAdam>
+__global__ void __launch_bounds__(256) k_weights(Adam q, Mats w) {
+    pdl_enter();
+    __shared__ __half tile[kWC][kWR + 2];
+    const int t = blockIdx.x;
+    if (t >= w.first[3]) {
+        if (!kAdam) return;
+        int e = (t - w.first[3]) * 256 + threadIdx.x;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            if (e >= 0 && e < w.nbias[l]) adam_one<kAdam>(q, w.off[2 * l + 1] + e);
+            e -= w.nbias[l];
+        }
+        return;
+    }
+    const int l = t >= w.first[2] ? 2 : (t >= w.first[1] ? 1 : 0);
+    const int rows = w.rows[l], cols = w.cols[l];
+    const int r0 = (t - w.first[l]) / w.tiles_c[l] * kWR, c0 = (t - w.first[l]) % w.tiles_c[l] * kWC;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < kWR; i += 8) {
+        const int r = r0 + ty + i, c = c0 + tx;
+        if (r < rows && c < cols) {
+            const __half h = __float2half_rn(adam_one<kAdam>(q, w.off[2 * l] + (size_t)r * cols + c));
+            if (w.wn[l]) w.wn[l][(size_t)r * w.ldn[l] + c] = h;
+            tile[tx][ty + i] = h;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kWC; i += 8) {
+        const int c = c0 + ty + i, r = r0 + 2 * tx;
+        if (c >= cols || r >= rows) continue;
+        __half* d = w.wt[l] + (size_t)c * w.ldt[l] + r;
+        if (r + 1 < rows) *reinterpret_cast<__half2*>(d) = *reinterpret_cast<const __half2*>(&tile[ty + i][2 * tx]);
+        else *d = tile[ty + i][2 * tx];
     }
 }
 
@@ -147,14 +312,14 @@ struct lp_mlp {
     __half *w1t = nullptr, *w2t = nullptr, *w3t = nullptr;           // W^T: [hid x in], [hid x hid], [out x hid]
     __half *w2n = nullptr, *w3n = nullptr;                           // W:   [hid x hid], [hid x out]
     __half *x16 = nullptr, *xT = nullptr;                            // [maxb x in], [in x maxb]
-    float *z1 = nullptr, *z2 = nullptr, *z3 = nullptr;               // pre-activations
+    float *z1 = nullptr, *z2 = nullptr;                              // pre-activations
     __half *a1 = nullptr, *a2 = nullptr, *a1T = nullptr, *a2T = nullptr;
     __half *dz3 = nullptr, *dz2 = nullptr, *dz1 = nullptr;
     __half *dz3T = nullptr, *dz2T = nullptr, *dz1T = nullptr;
-    float *da2 = nullptr, *da1 = nullptr;
     float* loss = nullptr;
     int32_t* err = nullptr;  // bounded-wait flag of the tensor-core GEMMs
     int64_t steps = 0;
+    int sms = 1;
 };
 
 namespace {
@@ -177,74 +342,100 @@ int malloc_t(lp_mlp* h, T** p, size_t n) {
     return LP_OK;
 }
 
-// D (M x N, FP32, row stride ldd) = X (M x K, FP16, row stride ldx) * Y (N x K, FP16, row stride ldy)^T
-int gemm(const lp_mlp* h, int M, int N, int K, const __half* X, int ldx, const __half* Y, int ldy, float* D,
-         int ldd) {
-    MCK(lpgb::tc_gemm(X, ldx, Y, ldy, D, ldd, M, N, K, false, h->err, h->stream));
+// epi(X Y^T): X is M x K (row stride ldx), Y N x K (row stride ldy), both FP16.
+// Tiles of 32 columns while the chip holds them at once, else 64, else 128; the
+// deeper rings of the narrow tiles keep as many bytes in flight.
+template <class Epi>
+int gemm(const lp_mlp* h, int M, int N, int K, const __half* X, int ldx, const __half* Y, int ldy, const Epi& epi) {
+    using namespace lpgb;
+    const int mt = (M + tcg::kTM - 1) / tcg::kTM;
+    const int bn = mt * ((N + 31) / 32) <= h->sms ? 32 : (mt * ((N + 63) / 64) <= h->sms ? 64 : 128);
+    const int ar = M >= tcg::kTM ? tcg::kTM : (M + 7) & ~7;  // whole 8-row swizzle atoms
+    CUtensorMap ma, mb;
+    if (!tc_make_map_16bit(&ma, X, M, K, ldx, ar, false) || !tc_make_map_16bit(&mb, Y, N, K, ldy, bn, false))
+        return LP_ERR_CUDA;
+    cudaError_t e;
+    if (bn == 32) e = tcg::launch_tc_gemm<32, 10, 1, false>(ma, mb, epi, M, N, K, ar, h->err, h->stream, true);
+    else if (bn == 64) e = tcg::launch_tc_gemm<64, 8, 1, false>(ma, mb, epi, M, N, K, ar, h->err, h->stream, true);
+    else e = tcg::launch_tc_gemm<128, 6, 1, false>(ma, mb, epi, M, N, K, ar, h->err, h->stream, true);
+    MCK(e);
     return LP_OK;
 }
 
-int blocks_for(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 4096); }
-
-// FP16 copies of the weights from the FP32 masters
-int refresh_weights(lp_mlp* h) {
-    const float *W1 = h->p + h->off[0], *W2 = h->p + h->off[2], *W3 = h->p + h->off[4];
-    k_weight16<<<blocks_for((size_t)h->in * h->hid), 256, 0, h->stream>>>(W1, h->in, h->hid, nullptr, 0, h->w1t, h->in_p);
-    k_weight16<<<blocks_for((size_t)h->hid * h->hid), 256, 0, h->stream>>>(W2, h->hid, h->hid, h->w2n, h->hid_p, h->w2t,
-                                                                            h->hid_p);
-    k_weight16<<<blocks_for((size_t)h->hid * h->out), 256, 0, h->stream>>>(W3, h->hid, h->out, h->w3n, h->out_p, h->w3t,
-                                                                            h->hid_p);
-    MCK(cudaGetLastError());
+// One Adam step with the gradients in h->g (lr > 0) and the FP16 weights, or the weights alone
+int refresh_weights(lp_mlp* h, float lr = 0.f) {
+    Mats w{};
+    const int in[3] = {h->in, h->hid, h->hid}, out[3] = {h->hid, h->hid, h->out};
+    __half* wn[3] = {nullptr, h->w2n, h->w3n};
+    __half* wt[3] = {h->w1t, h->w2t, h->w3t};
+    int biases = 0;
+    for (int l = 0; l < 3; ++l) {
+        w.rows[l] = in[l];
+        w.cols[l] = out[l];
+        w.tiles_c[l] = (out[l] + kWC - 1) / kWC;
+        w.first[l + 1] = w.first[l] + w.tiles_c[l] * ((in[l] + kWR - 1) / kWR);
+        w.off[2 * l] = h->off[2 * l];
+        w.off[2 * l + 1] = h->off[2 * l + 1];
+        w.nbias[l] = out[l];
+        w.wn[l] = wn[l];
+        w.wt[l] = wt[l];
+        w.ldn[l] = l == 2 ? h->out_p : h->hid_p;
+        w.ldt[l] = l == 0 ? h->in_p : h->hid_p;
+        biases += out[l];
+    }
+    Adam q{h->p, h->m1, h->m2, h->g, lr, 0.9f, 0.999f, 1e-8f, 1.f, 1.f};
+    if (lr > 0.f) {
+        q.c1 = 1.f - powf(q.b1, (float)h->steps);
+        q.c2 = 1.f - powf(q.b2, (float)h->steps);
+        MCK(launch_k(k_weights<true>, dim3(w.first[3] + (biases + 255) / 256), dim3(256), 0, h->stream, true, q, w));
+    } else {
+        MCK(launch_k(k_weights<false>, dim3(w.first[3]), dim3(256), 0, h->stream, false, q, w));
+    }
     return LP_OK;
 }
 
-// forward pass for a batch already converted to x16 / xT; logits in z3
-int forward(lp_mlp* h, int B) {
-    const float *b1 = h->p + h->off[1], *b2 = h->p + h->off[3], *b3 = h->p + h->off[5];
+// the hidden layers for a batch already in x16; back: what the backward pass reads is kept too
+int hidden_layers(lp_mlp* h, int B, bool back) {
+    const float *b1 = h->p + h->off[1], *b2 = h->p + h->off[3];
     int rc;
-    if ((rc = gemm(h, B, h->hid, h->in, h->x16, h->in_p, h->w1t, h->in_p, h->z1, h->hid))) return rc;
-    k_bias_act<<<blocks_for((size_t)B * h->hid), 256, 0, h->stream>>>(h->z1, b1, B, h->hid, 1, h->a1, h->hid_p, h->a1T,
-                                                                      h->b_p);
-    if ((rc = gemm(h, B, h->hid, h->hid, h->a1, h->hid_p, h->w2t, h->hid_p, h->z2, h->hid))) return rc;
-    k_bias_act<<<blocks_for((size_t)B * h->hid), 256, 0, h->stream>>>(h->z2, b2, B, h->hid, 1, h->a2, h->hid_p, h->a2T,
-                                                                      h->b_p);
-    if ((rc = gemm(h, B, h->out, h->hid, h->a2, h->hid_p, h->w3t, h->hid_p, h->z3, h->out))) return rc;
-    k_bias_act<<<blocks_for((size_t)B * h->out), 256, 0, h->stream>>>(h->z3, b3, B, h->out, 0, nullptr, 0, nullptr, 0);
-    MCK(cudaGetLastError());
-    return LP_OK;
+    if ((rc = gemm(h, B, h->hid, h->in, h->x16, h->in_p, h->w1t, h->in_p,
+                   EpiAct{b1, back ? h->z1 : nullptr, h->a1, back ? h->a1T : nullptr, h->hid_p, h->b_p, B, h->hid})))
+        return rc;
+    return gemm(h, B, h->hid, h->hid, h->a1, h->hid_p, h->w2t, h->hid_p,
+                EpiAct{b2, back ? h->z2 : nullptr, h->a2, back ? h->a2T : nullptr, h->hid_p, h->b_p, B, h->hid});
 }
 
 // loss and gradients into h->g for targets t (fp32, device, [B x out])
-int backward(lp_mlp* h, int B, const float* t) {
-    MCK(cudaMemsetAsync(h->loss, 0, sizeof(float), h->stream));
-    k_bce<<<blocks_for((size_t)B * h->out), 256, 0, h->stream>>>(h->z3, t, B, h->out, h->dz3, h->out_p, h->dz3T, h->b_p,
-                                                                 h->loss);
-    float *gW1 = h->g + h->off[0], *gb1 = h->g + h->off[1], *gW2 = h->g + h->off[2];
-    float *gb2 = h->g + h->off[3], *gW3 = h->g + h->off[4], *gb3 = h->g + h->off[5];
+int forward_backward(lp_mlp* h, int B, const float* t) {
     int rc;
-    // layer 3: gW3 = a2^T dz3, da2 = dz3 W3^T
-    if ((rc = gemm(h, h->hid, h->out, B, h->a2T, h->b_p, h->dz3T, h->b_p, gW3, h->out))) return rc;
-    k_colsum<<<(h->out + 255) / 256, 256, 0, h->stream>>>(h->dz3, h->out_p, B, h->out, gb3);
-    if ((rc = gemm(h, B, h->hid, h->out, h->dz3, h->out_p, h->w3n, h->out_p, h->da2, h->hid))) return rc;
-    k_relu_back<<<blocks_for((size_t)B * h->hid), 256, 0, h->stream>>>(h->da2, h->z2, B, h->hid, h->dz2, h->hid_p,
-                                                                       h->dz2T, h->b_p);
-    // layer 2: gW2 = a1^T dz2, da1 = dz2 W2^T
-    if ((rc = gemm(h, h->hid, h->hid, B, h->a1T, h->b_p, h->dz2T, h->b_p, gW2, h->hid))) return rc;
-    k_colsum<<<(h->hid + 255) / 256, 256, 0, h->stream>>>(h->dz2, h->hid_p, B, h->hid, gb2);
-    if ((rc = gemm(h, B, h->hid, h->hid, h->dz2, h->hid_p, h->w2n, h->hid_p, h->da1, h->hid))) return rc;
-    k_relu_back<<<blocks_for((size_t)B * h->hid), 256, 0, h->stream>>>(h->da1, h->z1, B, h->hid, h->dz1, h->hid_p,
-                                                                       h->dz1T, h->b_p);
-    // layer 1: gW1 = x^T dz1
-    if ((rc = gemm(h, h->in, h->hid, B, h->xT, h->b_p, h->dz1T, h->b_p, gW1, h->hid))) return rc;
-    k_colsum<<<(h->hid + 255) / 256, 256, 0, h->stream>>>(h->dz1, h->hid_p, B, h->hid, gb1);
-    MCK(cudaGetLastError());
+    if ((rc = hidden_layers(h, B, true))) return rc;
+    // layer 3: dz3 and the loss with the logits; da2 = dz3 W3^T, dz2; da1 = dz2 W2^T, dz1
+    if ((rc = gemm(h, B, h->out, h->hid, h->a2, h->hid_p, h->w3t, h->hid_p,
+                   EpiBce{h->p + h->off[5], t, h->dz3, h->dz3T, h->loss, h->out_p, h->b_p, B, h->out})))
+        return rc;
+    if ((rc = gemm(h, B, h->hid, h->out, h->dz3, h->out_p, h->w3n, h->out_p,
+                   EpiReluBack{h->z2, h->dz2, h->dz2T, h->hid_p, h->b_p, B, h->hid})))
+        return rc;
+    if ((rc = gemm(h, B, h->hid, h->hid, h->dz2, h->hid_p, h->w2n, h->hid_p,
+                   EpiReluBack{h->z1, h->dz1, h->dz1T, h->hid_p, h->b_p, B, h->hid})))
+        return rc;
+    // gW3 = a2^T dz3, gW2 = a1^T dz2, gW1 = x^T dz1
+    if ((rc = gemm(h, h->hid, h->out, B, h->a2T, h->b_p, h->dz3T, h->b_p, EpiStore{h->g + h->off[4], h->hid, h->out})))
+        return rc;
+    if ((rc = gemm(h, h->hid, h->hid, B, h->a1T, h->b_p, h->dz2T, h->b_p, EpiStore{h->g + h->off[2], h->hid, h->hid})))
+        return rc;
+    if ((rc = gemm(h, h->in, h->hid, B, h->xT, h->b_p, h->dz1T, h->b_p, EpiStore{h->g + h->off[0], h->in, h->hid})))
+        return rc;
+    const ColSum q{{h->dz3, h->dz2, h->dz1}, {h->g + h->off[5], h->g + h->off[3], h->g + h->off[1]},
+                   {h->out_p, h->hid_p, h->hid_p}, {h->out, h->hid, h->hid}};
+    MCK(launch_k(k_colsum, dim3((std::max(h->out, h->hid) + 63) / 64, 3), dim3(64), 0, h->stream, true, q, B));
     return LP_OK;
 }
 
-int load_x(lp_mlp* h, const float* X, int B) {
+int load_x(lp_mlp* h, const float* X, int B, bool back) {
     if (B < 1 || B > h->maxb || !X) return LP_ERR_INVALID_ARG;
-    k_input16<<<blocks_for((size_t)B * h->in), 256, 0, h->stream>>>(X, B, h->in, h->x16, h->in_p, h->xT, h->b_p);
-    MCK(cudaGetLastError());
+    MCK(launch_k(k_input16, dim3((h->in + kTile - 1) / kTile, (B + kTile - 1) / kTile), dim3(256), 0, h->stream, false, X,
+                 B, h->in, h->x16, h->in_p, back ? h->xT : (__half*)nullptr, h->b_p, back ? h->loss : (float*)nullptr));
     return LP_OK;
 }
 
@@ -269,6 +460,12 @@ int lp_mlp_create(lp_mlp** out, int32_t in_dim, int32_t hidden, int32_t out_dim,
     h->in = in_dim; h->hid = hidden; h->out = out_dim; h->maxb = max_batch;
     h->in_p = pad8(in_dim); h->hid_p = pad8(hidden); h->out_p = pad8(out_dim); h->b_p = pad8(max_batch);
     h->stream = static_cast<cudaStream_t>(cuda_stream);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        delete h;
+        return LP_ERR_CUDA;
+    }
     const size_t sz[6] = {(size_t)in_dim * hidden, (size_t)hidden, (size_t)hidden * hidden, (size_t)hidden,
                           (size_t)hidden * out_dim, (size_t)out_dim};
     size_t o = 0;
@@ -281,13 +478,12 @@ int lp_mlp_create(lp_mlp** out, int32_t in_dim, int32_t hidden, int32_t out_dim,
         (rc = malloc_t(h, &h->w2t, H * h->hid_p)) || (rc = malloc_t(h, &h->w3t, O * h->hid_p)) ||
         (rc = malloc_t(h, &h->w2n, H * h->hid_p)) || (rc = malloc_t(h, &h->w3n, H * h->out_p)) ||
         (rc = malloc_t(h, &h->x16, B * h->in_p)) || (rc = malloc_t(h, &h->xT, I * h->b_p)) ||
-        (rc = malloc_t(h, &h->z1, B * H)) || (rc = malloc_t(h, &h->z2, B * H)) || (rc = malloc_t(h, &h->z3, B * O)) ||
+        (rc = malloc_t(h, &h->z1, B * H)) || (rc = malloc_t(h, &h->z2, B * H)) ||
         (rc = malloc_t(h, &h->a1, B * h->hid_p)) || (rc = malloc_t(h, &h->a2, B * h->hid_p)) ||
         (rc = malloc_t(h, &h->a1T, H * h->b_p)) || (rc = malloc_t(h, &h->a2T, H * h->b_p)) ||
         (rc = malloc_t(h, &h->dz3, B * h->out_p)) || (rc = malloc_t(h, &h->dz2, B * h->hid_p)) ||
         (rc = malloc_t(h, &h->dz1, B * h->hid_p)) || (rc = malloc_t(h, &h->dz3T, O * h->b_p)) ||
         (rc = malloc_t(h, &h->dz2T, H * h->b_p)) || (rc = malloc_t(h, &h->dz1T, H * h->b_p)) ||
-        (rc = malloc_t(h, &h->da2, B * H)) || (rc = malloc_t(h, &h->da1, B * H)) ||
         (rc = malloc_t(h, &h->loss, 1)) || (rc = malloc_t(h, &h->err, 1))) {
         lp_mlp_destroy(h);
         return rc;
@@ -325,20 +521,18 @@ int lp_mlp_get_params(const lp_mlp* h, float* params) {
 
 int lp_mlp_forward(lp_mlp* h, const float* X, int32_t batch, float* logits) {
     if (!h || !logits) return LP_ERR_INVALID_ARG;
-    int rc = load_x(h, X, batch);
+    int rc = load_x(h, X, batch, false);
     if (rc != LP_OK) return rc;
-    if ((rc = forward(h, batch)) != LP_OK) return rc;
-    MCK(cudaMemcpyAsync(logits, h->z3, (size_t)batch * h->out * sizeof(float), cudaMemcpyDeviceToDevice, h->stream));
-    MCK(cudaGetLastError());
-    return LP_OK;
+    if ((rc = hidden_layers(h, batch, false)) != LP_OK) return rc;
+    return gemm(h, batch, h->out, h->hid, h->a2, h->hid_p, h->w3t, h->hid_p,
+                EpiAct{h->p + h->off[5], logits, nullptr, nullptr, 0, 0, batch, h->out});
 }
 
 int lp_mlp_gradients(lp_mlp* h, const float* X, const float* T, int32_t batch, float* grads, float* loss) {
     if (!h || !T) return LP_ERR_INVALID_ARG;
-    int rc = load_x(h, X, batch);
+    int rc = load_x(h, X, batch, true);
     if (rc != LP_OK) return rc;
-    if ((rc = forward(h, batch)) != LP_OK) return rc;
-    if ((rc = backward(h, batch, T)) != LP_OK) return rc;
+    if ((rc = forward_backward(h, batch, T)) != LP_OK) return rc;
     if (grads) MCK(cudaMemcpyAsync(grads, h->g, h->np * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
     if (loss) MCK(cudaMemcpyAsync(loss, h->loss, sizeof(float), cudaMemcpyDeviceToHost, h->stream));
     return check_err(h);
@@ -346,16 +540,11 @@ int lp_mlp_gradients(lp_mlp* h, const float* X, const float* T, int32_t batch, f
 
 int lp_mlp_train_step(lp_mlp* h, const float* X, const float* T, int32_t batch, float lr, float* loss) {
     if (!h || !T || !(lr > 0.f)) return LP_ERR_INVALID_ARG;
-    int rc = load_x(h, X, batch);
+    int rc = load_x(h, X, batch, true);
     if (rc != LP_OK) return rc;
-    if ((rc = forward(h, batch)) != LP_OK) return rc;
-    if ((rc = backward(h, batch, T)) != LP_OK) return rc;
+    if ((rc = forward_backward(h, batch, T)) != LP_OK) return rc;
     h->steps++;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.f - powf(b1, (float)h->steps), c2 = 1.f - powf(b2, (float)h->steps);
-    k_adam<<<blocks_for(h->np), 256, 0, h->stream>>>(h->p, h->g, h->m1, h->m2, h->np, lr, b1, b2, 1e-8f, c1, c2);
-    MCK(cudaGetLastError());
-    if ((rc = refresh_weights(h)) != LP_OK) return rc;
+    if ((rc = refresh_weights(h, lr)) != LP_OK) return rc;
     if (loss) {
         MCK(cudaMemcpyAsync(loss, h->loss, sizeof(float), cudaMemcpyDeviceToHost, h->stream));
         return check_err(h);

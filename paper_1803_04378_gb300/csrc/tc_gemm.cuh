@@ -41,11 +41,14 @@ struct GemmSmem {
 // with the tile row of the lane (0..127, the TMEM lane), the tile's first row
 // and column in the output, the first of the 32 columns, and their values.
 // kStages shared-memory stages; kMinBlocks CTAs share an SM (their TMEM
-// allocations, BN columns each, must fit the SM's 512).
+// allocations, BN columns each, must fit the SM's 512).  a_rows: rows of the
+// A tile that the TMA loads (the box height of ma, at most 128).  With fewer
+// rows of A than 128 the rest of the tile is neither loaded nor read back: the
+// MMA's rows do not mix, so its other output rows hold values nobody uses.
 template <int BN, int kStages, int kMinBlocks, bool kBF16, class Epi>
 __global__ void __launch_bounds__(kGemmThreads, kMinBlocks)
     k_tc_gemm(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb, Epi epi, int K,
-              int32_t* err) {
+              int a_rows, int32_t* err) {
     static_assert(kMinBlocks * BN <= 512, "TMEM columns of the co-resident CTAs");
     using L = GemmSmem<BN, kStages>;
     extern __shared__ uint8_t smem_raw[];
@@ -72,11 +75,13 @@ __global__ void __launch_bounds__(kGemmThreads, kMinBlocks)
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tholder;
+    pdl_enter();  // (the setup above ran beside the previous launch's tail)
 
     if (warp == 0) {
         if (lane == 0) {
             tc::tma_prefetch_desc(&ma);
             tc::tma_prefetch_desc(&mb);
+            const uint32_t tx = (uint32_t)(a_rows * kTK * 2 + L::kB);
             for (int kb = 0; kb < nk; ++kb) {
                 const int s = kb % kStages, use = kb / kStages;
                 if (kb >= kStages && !tc::mbar_wait(&empty[s], (use - 1) & 1)) {
@@ -84,7 +89,7 @@ __global__ void __launch_bounds__(kGemmThreads, kMinBlocks)
                     break;
                 }
                 uint8_t* sa = smem + s * L::kStage;
-                tc::mbar_arrive_expect_tx(&full[s], L::kStage);
+                tc::mbar_arrive_expect_tx(&full[s], tx);
                 tc::tma_load_2d(sa, &ma, &full[s], kb * kTK, m0);
                 tc::tma_load_2d(sa + L::kA, &mb, &full[s], kb * kTK, n0);
             }
@@ -311,17 +316,19 @@ cudaError_t launch_tc_gemm_p(const CUtensorMap& ma, const CUtensorMap& mb, const
                     dim3(gemm_p_threads<kEpiWarps>()), L::kBytes, st, true, ma, mb, epi, M, N, K, err);
 }
 
-// Tensor maps of the two operands and the launch (grid = N/BN x M/128 tiles).
+// The launch (grid = N/BN x M/128 tiles), programmatic where the caller's chain is.
 template <int BN, int kStages, int kMinBlocks, bool kBF16, class Epi>
 cudaError_t launch_tc_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const Epi& epi, int M, int N, int K,
-                           int32_t* err, cudaStream_t st) {
+                           int a_rows, int32_t* err, cudaStream_t st, bool pdl) {
     using L = GemmSmem<BN, kStages>;
+    static_assert(L::kBars >= (2 * kStages + 1) * 8 + 4, "barrier area");
+    static_assert(kMinBlocks * (L::kBytes + 1024) <= 232448, "shared memory of the co-resident CTAs");
     static cudaError_t attr_rc = cudaFuncSetAttribute(k_tc_gemm<BN, kStages, kMinBlocks, kBF16, Epi>,
                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::kBytes);
     if (attr_rc != cudaSuccess) return attr_rc;
     const dim3 grid((N + BN - 1) / BN, (M + kTM - 1) / kTM);
-    k_tc_gemm<BN, kStages, kMinBlocks, kBF16, Epi><<<grid, kGemmThreads, L::kBytes, st>>>(ma, mb, epi, K, err);
-    return cudaGetLastError();
+    return launch_k(k_tc_gemm<BN, kStages, kMinBlocks, kBF16, Epi>, grid, dim3(kGemmThreads), L::kBytes, st, pdl, ma, mb,
+                    epi, K, a_rows, err);
 }
 
 }  // namespace tcg
