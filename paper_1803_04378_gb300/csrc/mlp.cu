@@ -14,11 +14,11 @@
 // FP16 operand is kept in the layout its GEMM reads: activations row-major
 // [B x features] and, for the weight gradients, transposed [features x B];
 // the weights as W^T (forward) and W (the input gradients of the backward
-// pass).  FP16 rows are padded to a multiple of 8 elements (16-byte TMA
-// strides); FP32 results keep the logical widths.  Parameters are packed
+// pass).  FP16 rows are padded with zeros to a multiple of 64 elements (whole K
+// blocks); FP32 results keep the logical widths.  Parameters are packed
 // W1, b1, W2, b2, W3, b3 with W_l row-major [in_l x out_l].
 //
-// The element-wise work rides in the GEMMs' epilogues: a lane of an epilogue
+// Bias, ReLU and its backward ride in the GEMMs' epilogues: a lane of an epilogue
 // warp holds 32 columns of one row, so the row-major copy leaves in 16-byte
 // stores and the transposed copy in 64-byte rows of a warp.  (As kernels of
 // their own, with the transposed copy written element by element, they took
@@ -45,7 +45,8 @@ using lpgb::pdl_enter;
 
 namespace {
 
-inline int pad8(int v) { return (v + 7) & ~7; }
+// FP16 row strides: whole K blocks of the GEMMs, the padding zero
+inline int pad64(int v) { return (v + 63) & ~63; }
 
 // 32 consecutive halves of row `row` from column c0 (row stride ld, a multiple
 // of 8, base 16-byte aligned): 16-byte stores where all columns exist
@@ -60,11 +61,13 @@ __device__ __forceinline__ void store_row16(__half* a, int ld, int row, int c0, 
             if (c0 + i < N) p[i] = h[i];
     }
 }
-// the same as column `row` of the transposed copy: a warp's rows side by side
-__device__ __forceinline__ void store_col16(__half* aT, int ldt, int row, int c0, int N, const __half (&h)[32]) {
+// the same as column `row` of the transposed copy: a warp's rows side by side; the
+// rows between M and the next multiple of 64 are zero (K of the weight gradients)
+__device__ __forceinline__ void store_col16(__half* aT, int ldt, int row, int M, int c0, int N, const __half (&h)[32]) {
+    if (row >= ((M + 63) & ~63)) return;
 #pragma unroll
     for (int i = 0; i < 32; ++i)
-        if (c0 + i < N) aT[(size_t)(c0 + i) * ldt + row] = h[i];
+        if (c0 + i < N) aT[(size_t)(c0 + i) * ldt + row] = row < M ? h[i] : __float2half_rn(0.f);
 }
 __device__ __forceinline__ void load_row32(const float* z, int ld, int row, int c0, int N, float (&v)[32]) {
     const float* p = z + (size_t)row * ld + c0;
@@ -100,7 +103,8 @@ struct EpiStore {
     }
 };
 
-// z = acc + bias; with a: a = relu(z) in FP16, and with aT its transpose; z itself where it is asked for
+// z = acc + bias; with a: a = relu(z) in FP16, and with aT its transpose; z itself
+// where it is asked for
 struct EpiAct {
     const float* bias;
     float* z;
@@ -108,53 +112,17 @@ struct EpiAct {
     int lda, ldt, M, N;
     __device__ void operator()(int trow, int m0, int n0, int c0, const float (&v)[32]) const {
         const int row = m0 + trow, c = n0 + c0;
-        if (row >= M) return;
         float x[32];
 #pragma unroll
         for (int i = 0; i < 32; ++i) x[i] = v[i] + (c + i < N ? __ldg(bias + c + i) : 0.f);
-        if (z) store_row32(z, N, row, c, N, x);
+        if (z && row < M) store_row32(z, N, row, c, N, x);
         if (a) {
             __align__(16) __half h[32];
 #pragma unroll
             for (int i = 0; i < 32; ++i) h[i] = __float2half_rn(fmaxf(x[i], 0.f));
-            store_row16(a, lda, row, c, N, h);
-            if (aT) store_col16(aT, ldt, row, c, N, h);
+            if (row < M) store_row16(a, lda, row, c, N, h);
+            if (aT) store_col16(aT, ldt, row, M, c, N, h);
         }
-    }
-};
-
-// z = acc + bias; dz = (sigmoid(z) - t) / B in FP16, row-major and transposed; the loss's partial sums
-// (softplus(z) - t z) / B
-struct EpiBce {
-    const float *bias, *t;
-    __half *dz, *dzT;
-    float* loss;
-    int ld, ldt, M, N;
-    __device__ void operator()(int trow, int m0, int n0, int c0, const float (&v)[32]) const {
-        const int row = m0 + trow, c = n0 + c0;
-        const float inv = 1.f / (float)M;
-        float l = 0.f;
-        if (row < M) {
-            float tt[32];
-            load_row32(t, N, row, c, N, tt);
-            __align__(16) __half h[32];
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                if (c + i < N) {
-                    const float x = v[i] + __ldg(bias + c + i);
-                    const float sp = x > 0.f ? x + log1pf(expf(-x)) : log1pf(expf(x));
-                    l += (sp - tt[i] * x) * inv;
-                    const float sg = 1.f / (1.f + expf(-x));
-                    h[i] = __float2half_rn((sg - tt[i]) * inv);
-                } else {
-                    h[i] = __float2half_rn(0.f);
-                }
-            }
-            store_row16(dz, ld, row, c, N, h);
-            store_col16(dzT, ldt, row, c, N, h);
-        }
-        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-        if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
     }
 };
 
@@ -165,71 +133,131 @@ struct EpiReluBack {
     int ld, ldt, M, N;
     __device__ void operator()(int trow, int m0, int n0, int c0, const float (&v)[32]) const {
         const int row = m0 + trow, c = n0 + c0;
-        if (row >= M) return;
-        float zz[32];
-        load_row32(z, N, row, c, N, zz);
         __align__(16) __half h[32];
+        if (row < M) {
+            float zz[32];
+            load_row32(z, N, row, c, N, zz);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) h[i] = __float2half_rn(zz[i] > 0.f ? v[i] : 0.f);
-        store_row16(dz, ld, row, c, N, h);
-        store_col16(dzT, ldt, row, c, N, h);
+            for (int i = 0; i < 32; ++i) h[i] = __float2half_rn(zz[i] > 0.f ? v[i] : 0.f);
+            store_row16(dz, ld, row, c, N, h);
+        }
+        store_col16(dzT, ldt, row, M, c, N, h);
     }
 };
 
 // X (rows x cols, FP32) -> x16 (row stride ld) and, where asked for, xT (cols x
-// rows, row stride ldt), FP16, by 32 x 32 tiles through shared memory; loss = 0
+// rows, row stride ldt, zero up to the next multiple of 64 rows), FP16, by 32 x 32
+// tiles through shared memory
 constexpr int kTile = 32;
 __global__ void __launch_bounds__(256) k_input16(const float* __restrict__ X, int rows, int cols,
-                                                 __half* __restrict__ x16, int ld, __half* __restrict__ xT, int ldt,
-                                                 float* loss) {
+                                                 __half* __restrict__ x16, int ld, __half* __restrict__ xT, int ldt) {
     pdl_enter();
     __shared__ __half tile[kTile][kTile + 2];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int c0 = blockIdx.x * kTile, r0 = blockIdx.y * kTile;
-    if (loss && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *loss = 0.f;
 #pragma unroll
     for (int i = 0; i < kTile; i += 8) {
         const int r = r0 + ty + i, c = c0 + tx;
+        __half h = __float2half_rn(0.f);
         if (r < rows && c < cols) {
-            const __half h = __float2half_rn(X[(size_t)r * cols + c]);
+            h = __float2half_rn(X[(size_t)r * cols + c]);
             x16[(size_t)r * ld + c] = h;
-            tile[ty + i][tx] = h;
         }
+        tile[ty + i][tx] = h;
     }
     if (!xT) return;
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < kTile; i += 8) {
         const int c = c0 + ty + i, r = r0 + tx;
-        if (r < rows && c < cols) xT[(size_t)c * ldt + r] = tile[tx][ty + i];
+        if (c < cols) xT[(size_t)c * ldt + r] = tile[tx][ty + i];  // (zero past the batch)
     }
 }
 
-// db[c] = sum_r dz[r][c], row by row, of the three layers' dz at once (32 rows of
-// loads in flight; one at a time the three sums took 55 us)
+// dz = (sigmoid(z) - t) / B in FP16 (row-major, and transposed with zeros up to the
+// next multiple of 64 rows); a partial sum per block of (softplus(z) - t z) / B.  32 x 32
+// tiles through shared memory; in the GEMM's epilogue the exponentials of 64 elements
+// per lane ran on four warps per SM and took 25 us at 256 x 3072, here 5.
+__global__ void __launch_bounds__(256) k_bce(const float* __restrict__ z, const float* __restrict__ t, int rows, int cols,
+                                             __half* __restrict__ dz, int ld, __half* __restrict__ dzT, int ldt,
+                                             float* __restrict__ part) {
+    pdl_enter();
+    __shared__ __half tile[kTile][kTile + 2];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int c0 = blockIdx.x * kTile, r0 = blockIdx.y * kTile;
+    const float inv = 1.f / (float)rows;
+    float l = 0.f;
+#pragma unroll
+    for (int i = 0; i < kTile; i += 8) {
+        const int r = r0 + ty + i, c = c0 + tx;
+        __half h = __float2half_rn(0.f);
+        if (r < rows && c < cols) {
+            const float v = z[(size_t)r * cols + c], tt = t[(size_t)r * cols + c];
+            const float sp = v > 0.f ? v + log1pf(expf(-v)) : log1pf(expf(v));
+            l += (sp - tt * v) * inv;
+            const float sg = 1.f / (1.f + expf(-v));
+            h = __float2half_rn((sg - tt) * inv);
+            dz[(size_t)r * ld + c] = h;
+        }
+        tile[ty + i][tx] = h;
+    }
+    __shared__ float wl[8];
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (tx == 0) wl[ty] = l;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) l += wl[w];
+        part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = l;
+    }
+#pragma unroll
+    for (int i = 0; i < kTile; i += 8) {
+        const int c = c0 + ty + i, r = r0 + tx;
+        if (c < cols) dzT[(size_t)c * ldt + r] = tile[tx][ty + i];
+    }
+}
+
+// db[c] = sum_r dz[r][c], row by row, of the three layers' dz at once: a block
+// loads 64 columns of 128 rows at a time and 64 of its threads add them (one
+// row's load in flight per column took the three sums 55 us, 32 rows 14)
+// The first block also adds the loss's partial sums, in a fixed order.
 struct ColSum {
     const __half* dz[3];
     float* db[3];
     int ld[3], cols[3];
+    const float* part;
+    int nparts;
+    float* loss;
 };
-__global__ void __launch_bounds__(64) k_colsum(ColSum q, int rows) {
+constexpr int kSumRows = 128, kSumCols = 64;
+__global__ void __launch_bounds__(256) k_colsum(ColSum q, int rows) {
     pdl_enter();
-    const int l = blockIdx.y;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= q.cols[l]) return;
-    const __half* p = q.dz[l] + c;
-    const size_t ld = q.ld[l];
-    float s = 0.f;
-    int r = 0;
-    for (; r + 32 <= rows; r += 32) {
-        __half h[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) h[i] = p[(r + i) * ld];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) s += __half2float(h[i]);
+    __shared__ __half tile[kSumRows][kSumCols];
+    const int l = blockIdx.y, c0 = blockIdx.x * kSumCols, tid = threadIdx.x;
+    if (l == 0 && c0 == 0 && tid < 32) {
+        double v = 0.0;
+        for (int e = tid; e < q.nparts; e += 32) v += (double)q.part[e];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (tid == 0) *q.loss = (float)v;
     }
-    for (; r < rows; ++r) s += __half2float(p[r * ld]);
-    q.db[l][c] = s;
+    if (c0 >= q.cols[l]) return;
+    float s = 0.f;
+    for (int r0 = 0; r0 < rows; r0 += kSumRows) {
+        const int nr = min(kSumRows, rows - r0);
+        // (rows are padded to 64 columns: whole 16-byte pieces)
+        for (int e = tid; e < nr * (kSumCols / 8); e += 256) {
+            const int r = e / (kSumCols / 8), c = 8 * (e % (kSumCols / 8));
+            *reinterpret_cast<uint4*>(&tile[r][c]) =
+                *reinterpret_cast<const uint4*>(q.dz[l] + (size_t)(r0 + r) * q.ld[l] + c0 + c);
+        }
+        __syncthreads();
+        if (tid < kSumCols) {
+            int r = 0;
+#pragma unroll 16
+            for (; r < nr; ++r) s += __half2float(tile[r][tid]);
+        }
+        __syncthreads();
+    }
+    if (tid < kSumCols && c0 + tid < q.cols[l]) q.db[l][c0 + tid] = s;
 }
 
 // One Adam step on every parameter (kAdam) and the FP16 copies of the weights from
@@ -303,7 +331,7 @@ __global__ void __launch_bounds__(256) k_weights(Adam q, Mats w) {
 
 struct lp_mlp {
     int in = 0, hid = 0, out = 0, maxb = 0;
-    int in_p = 0, hid_p = 0, out_p = 0, b_p = 0;  // FP16 row strides (multiples of 8)
+    int in_p = 0, hid_p = 0, out_p = 0, b_p = 0;  // FP16 row strides (multiples of 64)
     size_t np = 0;
     size_t off[6] = {};  // W1 b1 W2 b2 W3 b3 offsets into the packed vectors
     cudaStream_t stream = nullptr;
@@ -312,11 +340,12 @@ struct lp_mlp {
     __half *w1t = nullptr, *w2t = nullptr, *w3t = nullptr;           // W^T: [hid x in], [hid x hid], [out x hid]
     __half *w2n = nullptr, *w3n = nullptr;                           // W:   [hid x hid], [hid x out]
     __half *x16 = nullptr, *xT = nullptr;                            // [maxb x in], [in x maxb]
-    float *z1 = nullptr, *z2 = nullptr;                              // pre-activations
+    float *z1 = nullptr, *z2 = nullptr, *z3 = nullptr;               // pre-activations
     __half *a1 = nullptr, *a2 = nullptr, *a1T = nullptr, *a2T = nullptr;
     __half *dz3 = nullptr, *dz2 = nullptr, *dz1 = nullptr;
     __half *dz3T = nullptr, *dz2T = nullptr, *dz1T = nullptr;
     float* loss = nullptr;
+    float* part = nullptr;   // its partial sums, one per block of k_bce
     int32_t* err = nullptr;  // bounded-wait flag of the tensor-core GEMMs
     int64_t steps = 0;
     int sms = 1;
@@ -352,12 +381,13 @@ int gemm(const lp_mlp* h, int M, int N, int K, const __half* X, int ldx, const _
     const int bn = mt * ((N + 31) / 32) <= h->sms ? 32 : (mt * ((N + 63) / 64) <= h->sms ? 64 : 128);
     const int ar = M >= tcg::kTM ? tcg::kTM : (M + 7) & ~7;  // whole 8-row swizzle atoms
     CUtensorMap ma, mb;
-    if (!tc_make_map_16bit(&ma, X, M, K, ldx, ar, false) || !tc_make_map_16bit(&mb, Y, N, K, ldy, bn, false))
+    const int kb = bn == 32 ? tcg::GemmStage<32>::KB : (bn == 64 ? tcg::GemmStage<64>::KB : tcg::GemmStage<128>::KB);
+    if (!tc_make_map_16bit_k(&ma, X, M, K, ldx, ar, kb, false) || !tc_make_map_16bit_k(&mb, Y, N, K, ldy, bn, kb, false))
         return LP_ERR_CUDA;
     cudaError_t e;
-    if (bn == 32) e = tcg::launch_tc_gemm<32, 10, 1, false>(ma, mb, epi, M, N, K, ar, h->err, h->stream, true);
-    else if (bn == 64) e = tcg::launch_tc_gemm<64, 8, 1, false>(ma, mb, epi, M, N, K, ar, h->err, h->stream, true);
-    else e = tcg::launch_tc_gemm<128, 6, 1, false>(ma, mb, epi, M, N, K, ar, h->err, h->stream, true);
+    if (bn == 32) e = tcg::launch_tc_gemm<32, false, true>(ma, mb, epi, M, N, K, ar, h->err, h->stream, true);
+    else if (bn == 64) e = tcg::launch_tc_gemm<64, false, true>(ma, mb, epi, M, N, K, ar, h->err, h->stream, true);
+    else e = tcg::launch_tc_gemm<128, false, true>(ma, mb, epi, M, N, K, ar, h->err, h->stream, true);
     MCK(e);
     return LP_OK;
 }
@@ -409,10 +439,12 @@ int hidden_layers(lp_mlp* h, int B, bool back) {
 int forward_backward(lp_mlp* h, int B, const float* t) {
     int rc;
     if ((rc = hidden_layers(h, B, true))) return rc;
-    // layer 3: dz3 and the loss with the logits; da2 = dz3 W3^T, dz2; da1 = dz2 W2^T, dz1
+    // layer 3: logits, dz3 and the loss; da2 = dz3 W3^T, dz2; da1 = dz2 W2^T, dz1
     if ((rc = gemm(h, B, h->out, h->hid, h->a2, h->hid_p, h->w3t, h->hid_p,
-                   EpiBce{h->p + h->off[5], t, h->dz3, h->dz3T, h->loss, h->out_p, h->b_p, B, h->out})))
+                   EpiAct{h->p + h->off[5], h->z3, nullptr, nullptr, 0, 0, B, h->out})))
         return rc;
+    MCK(launch_k(k_bce, dim3((h->out + kTile - 1) / kTile, pad64(B) / kTile), dim3(256), 0, h->stream, true,
+                 (const float*)h->z3, t, B, h->out, h->dz3, h->out_p, h->dz3T, h->b_p, h->part));
     if ((rc = gemm(h, B, h->hid, h->out, h->dz3, h->out_p, h->w3n, h->out_p,
                    EpiReluBack{h->z2, h->dz2, h->dz2T, h->hid_p, h->b_p, B, h->hid})))
         return rc;
@@ -427,15 +459,16 @@ int forward_backward(lp_mlp* h, int B, const float* t) {
     if ((rc = gemm(h, h->in, h->hid, B, h->xT, h->b_p, h->dz1T, h->b_p, EpiStore{h->g + h->off[0], h->in, h->hid})))
         return rc;
     const ColSum q{{h->dz3, h->dz2, h->dz1}, {h->g + h->off[5], h->g + h->off[3], h->g + h->off[1]},
-                   {h->out_p, h->hid_p, h->hid_p}, {h->out, h->hid, h->hid}};
-    MCK(launch_k(k_colsum, dim3((std::max(h->out, h->hid) + 63) / 64, 3), dim3(64), 0, h->stream, true, q, B));
+                   {h->out_p, h->hid_p, h->hid_p}, {h->out, h->hid, h->hid}, h->part,
+                   (h->out + kTile - 1) / kTile * (pad64(B) / kTile), h->loss};
+    MCK(launch_k(k_colsum, dim3((std::max(h->out, h->hid) + kSumCols - 1) / kSumCols, 3), dim3(256), 0, h->stream, true, q, B));
     return LP_OK;
 }
 
 int load_x(lp_mlp* h, const float* X, int B, bool back) {
     if (B < 1 || B > h->maxb || !X) return LP_ERR_INVALID_ARG;
-    MCK(launch_k(k_input16, dim3((h->in + kTile - 1) / kTile, (B + kTile - 1) / kTile), dim3(256), 0, h->stream, false, X,
-                 B, h->in, h->x16, h->in_p, back ? h->xT : (__half*)nullptr, h->b_p, back ? h->loss : (float*)nullptr));
+    MCK(launch_k(k_input16, dim3((h->in + kTile - 1) / kTile, pad64(B) / kTile), dim3(256), 0, h->stream, false, X,
+                 B, h->in, h->x16, h->in_p, back ? h->xT : (__half*)nullptr, h->b_p));
     return LP_OK;
 }
 
@@ -458,7 +491,7 @@ int lp_mlp_create(lp_mlp** out, int32_t in_dim, int32_t hidden, int32_t out_dim,
     lp_mlp* h = new (std::nothrow) lp_mlp();
     if (!h) return LP_ERR_OOM;
     h->in = in_dim; h->hid = hidden; h->out = out_dim; h->maxb = max_batch;
-    h->in_p = pad8(in_dim); h->hid_p = pad8(hidden); h->out_p = pad8(out_dim); h->b_p = pad8(max_batch);
+    h->in_p = pad64(in_dim); h->hid_p = pad64(hidden); h->out_p = pad64(out_dim); h->b_p = pad64(max_batch);
     h->stream = static_cast<cudaStream_t>(cuda_stream);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -478,19 +511,30 @@ int lp_mlp_create(lp_mlp** out, int32_t in_dim, int32_t hidden, int32_t out_dim,
         (rc = malloc_t(h, &h->w2t, H * h->hid_p)) || (rc = malloc_t(h, &h->w3t, O * h->hid_p)) ||
         (rc = malloc_t(h, &h->w2n, H * h->hid_p)) || (rc = malloc_t(h, &h->w3n, H * h->out_p)) ||
         (rc = malloc_t(h, &h->x16, B * h->in_p)) || (rc = malloc_t(h, &h->xT, I * h->b_p)) ||
-        (rc = malloc_t(h, &h->z1, B * H)) || (rc = malloc_t(h, &h->z2, B * H)) ||
+        (rc = malloc_t(h, &h->z1, B * H)) || (rc = malloc_t(h, &h->z2, B * H)) || (rc = malloc_t(h, &h->z3, B * O)) ||
         (rc = malloc_t(h, &h->a1, B * h->hid_p)) || (rc = malloc_t(h, &h->a2, B * h->hid_p)) ||
         (rc = malloc_t(h, &h->a1T, H * h->b_p)) || (rc = malloc_t(h, &h->a2T, H * h->b_p)) ||
         (rc = malloc_t(h, &h->dz3, B * h->out_p)) || (rc = malloc_t(h, &h->dz2, B * h->hid_p)) ||
         (rc = malloc_t(h, &h->dz1, B * h->hid_p)) || (rc = malloc_t(h, &h->dz3T, O * h->b_p)) ||
         (rc = malloc_t(h, &h->dz2T, H * h->b_p)) || (rc = malloc_t(h, &h->dz1T, H * h->b_p)) ||
+        (rc = malloc_t(h, &h->part, ((O + kTile - 1) / kTile) * (h->b_p / kTile))) ||
         (rc = malloc_t(h, &h->loss, 1)) || (rc = malloc_t(h, &h->err, 1))) {
         lp_mlp_destroy(h);
         return rc;
     }
-    if (cudaMemsetAsync(h->p, 0, o * sizeof(float), h->stream) || cudaMemsetAsync(h->m1, 0, o * sizeof(float), h->stream) ||
-        cudaMemsetAsync(h->m2, 0, o * sizeof(float), h->stream) || cudaMemsetAsync(h->err, 0, sizeof(int32_t), h->stream) ||
-        refresh_weights(h) != LP_OK) {
+    bool ok = cudaMemsetAsync(h->p, 0, o * sizeof(float), h->stream) == cudaSuccess &&
+              cudaMemsetAsync(h->m1, 0, o * sizeof(float), h->stream) == cudaSuccess &&
+              cudaMemsetAsync(h->m2, 0, o * sizeof(float), h->stream) == cudaSuccess &&
+              cudaMemsetAsync(h->err, 0, sizeof(int32_t), h->stream) == cudaSuccess;
+    // the padding of the FP16 rows stays zero from here on
+    const struct { __half* p; size_t n; } padded[] = {
+        {h->w1t, H * h->in_p}, {h->w2t, H * h->hid_p}, {h->w3t, O * h->hid_p}, {h->w2n, H * h->hid_p},
+        {h->w3n, H * h->out_p}, {h->x16, B * h->in_p}, {h->xT, I * h->b_p}, {h->a1, B * h->hid_p},
+        {h->a2, B * h->hid_p}, {h->a1T, H * h->b_p}, {h->a2T, H * h->b_p}, {h->dz3, B * h->out_p},
+        {h->dz2, B * h->hid_p}, {h->dz1, B * h->hid_p}, {h->dz3T, O * h->b_p}, {h->dz2T, H * h->b_p},
+        {h->dz1T, H * h->b_p}};
+    for (const auto& q : padded) ok = ok && cudaMemsetAsync(q.p, 0, q.n * sizeof(__half), h->stream) == cudaSuccess;
+    if (!ok || refresh_weights(h) != LP_OK) {
         lp_mlp_destroy(h);
         return LP_ERR_CUDA;
     }

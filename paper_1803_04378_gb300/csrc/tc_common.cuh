@@ -70,6 +70,26 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
         : "memory");
 }
 
+// 3-D form: z counts blocks of 64 columns, so that one load brings several K blocks,
+// each a whole swizzled tile (tc_make_map_16bit_k).
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y, int z) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+            smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+        : "memory");
+}
+
+// One lane of a converged warp, the same one at every call.  A role's loop runs in all
+// 32 lanes and only the issue of a load, an MMA or a commit is elected: in a loop
+// of one lane the compiler moves every operand of an issue to the uniform
+// registers anew (75 cycles per MMA, 250 per pair of loads; 30 and 90 this way).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // ---- TMEM ------------------------------------------------------------------------
 // One full warp allocates `ncols` (a power of two >= 32) columns; the TMEM
 // address is written to *holder (shared memory).
@@ -155,5 +175,10 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 // aligned), box = box_rows x 64 elements with the 128-byte swizzle; elements
 // outside the matrix read as zero.  Returns false when cuTensorMapEncodeTiled rejects it.
 bool tc_make_map_16bit(CUtensorMap* map, const void* base, int rows, int cols, int ld, int box_rows, bool bf16);
+// The same matrix as ceil(cols / 64) blocks of 64 columns (x: within a block, y: row,
+// z: block), box = kblocks x box_rows x 64.  Reads up to the next multiple of
+// 64 columns, which must lie within the row and be zero.
+bool tc_make_map_16bit_k(CUtensorMap* map, const void* base, int rows, int cols, int ld, int box_rows, int kblocks,
+                         bool bf16);
 
 }  // namespace lpgb

@@ -68,6 +68,23 @@ bool tc_make_map_16bit(CUtensorMap* map, const void* base, int rows, int cols, i
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool tc_make_map_16bit_k(CUtensorMap* map, const void* base, int rows, int cols, int ld, int box_rows, int kblocks,
+                         bool bf16) {
+    EncodeTiledFn fn = encode_fn();
+    const int nk = (cols + tcg::kTK - 1) / tcg::kTK;
+    if (!fn || rows < 1 || cols < 1 || ld < nk * tcg::kTK || (ld % 8) != 0 || box_rows < 1 || box_rows > 256 ||
+        kblocks < 1 || (reinterpret_cast<uintptr_t>(base) & 15) != 0)
+        return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)tcg::kTK, (cuuint64_t)rows, (cuuint64_t)nk};
+    const cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)tcg::kTK * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)tcg::kTK, (cuuint32_t)box_rows, (cuuint32_t)kblocks};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3,
+              const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // D (M x N, FP32, row stride ldd) = A (M x K, row stride lda) * B (N x K, row
 // stride ldb)^T; 16-bit operands, lda and ldb multiples of 8, bases 16-byte
 // aligned.  Returns cudaErrorInvalidValue for shapes or pointers the tensor
@@ -80,8 +97,8 @@ cudaError_t tc_gemm(const void* A, int lda, const void* B, int ldb, float* D, in
     if (!tc_make_map_16bit(&ma, A, M, K, lda, tcg::kTM, bf16) || !tc_make_map_16bit(&mb, B, N, K, ldb, BN, bf16))
         return cudaErrorInvalidValue;
     const StoreF32 epi{D, ldd, M, N};
-    return bf16 ? tcg::launch_tc_gemm<BN, 4, 1, true>(ma, mb, epi, M, N, K, tcg::kTM, err, st, false)
-                : tcg::launch_tc_gemm<BN, 4, 1, false>(ma, mb, epi, M, N, K, tcg::kTM, err, st, false);
+    return bf16 ? tcg::launch_tc_gemm<BN, true, false>(ma, mb, epi, M, N, K, tcg::kTM, err, st, false)
+                : tcg::launch_tc_gemm<BN, false, false>(ma, mb, epi, M, N, K, tcg::kTM, err, st, false);
 }
 
 }  // namespace lpgb
