@@ -304,7 +304,9 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
     __shared__ double rinv_sh, cq_sh, thr_sh, dpart[2], cd[kRCand];
     __shared__ int screen_sh;
     __shared__ unsigned pub[2 * kRList];
-    __shared__ int bL, bcnt, bov, nrow, scan_sh;  // the CTA's PRICE record; the ratio test needs a scan
+    __shared__ int rep_sh, rep_code, rep_end, rep_row;  // warm-start repair: running, outcome
+    __shared__ double rep_val;
+    __shared__ int bL, bcnt, bov, nrow, scan_sh;  // the CTA's PRICE record; rows taken by the update; scan
     __shared__ int wL[kRPrice], wov[kRPrice], wn[kRPrice];          // PRICE meeting, per polling warp
     __shared__ int wlj[kRPrice][kRWarpList], wlh[kRPrice][kRWarpList];
     __shared__ int cl[kRCand];
@@ -327,7 +329,11 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
         S.z = C->z; S.bytes_price = C->bytes_price; S.bytes_update = C->bytes_update;
         S.k = C->k_live; S.par = C->map_par;
         screen_sh = P.screen && C->screen_off == 0;
+        rep_sh = C->repair == 1;
+        rep_code = 0;
     }
+    const double rep_tol = C->repair_tol;
+    const int rep_limit = C->repair_limit;
     __syncthreads();
     const int par = S.par;
     {
@@ -604,6 +610,125 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
                 }
             }
             break;
+        }
+        if (rep_sh) {
+            // ---- a warm-start repair pivot (k_repair_pick's rule): the most negative
+            // basic value leaves (ties: the smallest position) and the live slot with
+            // the most negative entry of its row enters (ties: the smallest row).  The
+            // entering column is a live column, so there is no FTRAN, and one meeting
+            // does.
+            if (piv) {
+                move_rows(tid, kRThreads);
+                apply_rows(r);
+            }
+            __syncthreads();
+            ++seq;
+            if (warp == 0) {
+                const long long klim = dkey(-rep_tol);
+                long long kb = kbig;
+                int pi = INT_MAX, var = 0;
+                for (int l = lane; l < owned; l += 32) {
+                    const long long key = dkey(bb[l]);
+                    if (key < klim && key < kb) { kb = key; pi = b + G * l; var = rvar[l]; }
+                }
+                const long long wm = warp_min_key(kb);
+                const int win = warp_argmin_index(pi, kb == wm && wm != kbig);
+                if (lane == 0) __threadfence();  // the updated rows, before the record
+                __syncwarp();
+                if (lane == max(win, 0)) {
+                    meet_put(xbuf, seq, 0, ll_lo(wm), ll_hi(wm), (unsigned)(win < 0 ? -1 : pi));
+                    meet_put(xbuf, seq, 1, 0, 0, (unsigned)var);
+                }
+            }
+            if (warp < nwu) {
+                unsigned w[kRWords];
+                long long kb = kbig;
+                int pi = INT_MAX, var = 0;
+                if (tid < G) {
+                    meet_get<0, 2>(xbuf, seq, tid, w, &fail);
+                    kb = words_ll(w[0], w[1]);
+                    pi = (int)w[2];
+                    var = (int)w[5];
+                }
+                const long long wm = warp_min_key(kb);
+                const int win = warp_argmin_index(pi, kb == wm && wm != kbig);
+                if (lane == max(win, 0)) { wmin[warp] = wm; wrow[warp] = win < 0 ? -1 : pi; wvar[warp] = var; }
+            }
+            __syncthreads();
+            if (fail) break;
+            int gw = 0;
+            for (int w = 1; w < nwu; ++w)
+                if (wmin[w] < wmin[gw] || (wmin[w] == wmin[gw] && wmin[w] != kbig && wrow[w] < wrow[gw])) gw = w;
+            const int p = wmin[gw] == kbig ? -1 : wrow[gw], pvar = wvar[gw];
+            const double pval = kdouble(wmin[gw]);
+            // row r once every CTA has read it
+            if (piv) apply_row_r(r);
+            if (p < 0 || S.it >= rep_limit) {
+                __syncthreads();
+                if (tid == 0) {
+                    rep_code = p < 0 ? 2 : 4;
+                    rep_end = S.it;
+                    rep_sh = 0;
+                    S.r = S.q = -1;
+                    S.pending = 0;
+                }
+                __syncthreads();
+                if (rep_code == 2) continue;  // feasible: the method goes on from here
+                break;
+            }
+            long long ek = kbig;
+            int er = INT_MAX;
+            for (int t = tid; t < kn; t += kRThreads) {
+                const long long key = dkey(__ldcg(s.bp + (size_t)p * ld + t));
+                const int row = sr[t];
+                if (key < 0 && (key < ek || (key == ek && row < er))) { ek = key; er = row; }
+            }
+            const long long wm = warp_min_key(ek);
+            const int win = warp_argmin_index(er, ek == wm && wm != kbig);
+            if (lane == max(win, 0)) { wcand[warp].d_all = wm; wcand[warp].j_all = win < 0 ? -1 : er; }
+            __syncthreads();
+            if (tid == 0) {
+                long long km = kbig;
+                int jr = -1;
+                for (int w = 0; w < kRWarps; ++w)
+                    if (wcand[w].j_all >= 0 &&
+                        (jr < 0 || wcand[w].d_all < km || (wcand[w].d_all == km && wcand[w].j_all < jr))) {
+                        km = wcand[w].d_all;
+                        jr = wcand[w].j_all;
+                    }
+                rep_row = jr;
+                rep_val = kdouble(km);
+            }
+            __syncthreads();
+            if (rep_row < 0) {
+                // no slack can repair the row
+                if (tid == 0) {
+                    rep_code = 3;
+                    rep_end = S.it;
+                    S.r = S.q = -1;
+                    S.pending = 0;
+                }
+                break;
+            }
+            const int es = rs[rep_row];
+            double* anxt = s.alpha + (size_t)(S.abuf ^ 1) * ld;
+            for (int l = tid; l < owned; l += kRThreads) {
+                const int i = b + G * l;
+                const double v = kB ? Bs[(size_t)l * kc + es] : __ldcg(s.bp + (size_t)i * ld + es);
+                al[l] = v;
+                anxt[i] = v;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                S.q = n + rep_row; S.r = p; S.leave = pvar;
+                S.dq = -ycur[es];
+                S.theta = pval / rep_val;
+                S.alpha_r = rep_val;
+                S.tcount = 1; S.flags = 0; S.pending = 0;
+                S.abuf ^= 1;
+            }
+            __syncthreads();
+            continue;
         }
         // ---- PRICE + CHUZC
         const bool bland = S.bland != 0;
@@ -1079,6 +1204,10 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
             for (int t = tid; t < ld; t += kRThreads) s.yp[(size_t)par * ld + t] = t < kn ? ycur[t] : 0.0;
         if (tid == 0) {
             iterate_flush(s, S);
+            if (rep_code) {
+                C->repair = rep_code;
+                C->repair_end = rep_end;
+            }
             if (fail) C->err = kErrTimeout;
         }
     }

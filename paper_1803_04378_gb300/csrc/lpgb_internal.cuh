@@ -108,6 +108,8 @@ struct Ctrl {
     int32_t refine_rej;    // reinversion by refinement: the residual was above the tolerance (the
                            // rebuild is discarded and redone by elimination)
     int32_t ticket_reinv;  // last-block ticket of k_reinv_finish (reset by the last block)
+    int32_t repair_end;    // warm-start repair in k_iterate_r: the iteration count when it ended
+    int32_t pad_;
 };
 
 // Per-CTA ratio-test record of k_iterate: the CTA's smallest ratio, and its

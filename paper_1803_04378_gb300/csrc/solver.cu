@@ -500,19 +500,28 @@ int reinvert(lp_handle* h, int check_feasible, bool refine, bool to_struct = fal
     return LP_OK;
 }
 
-// Up to graph_iters + 1 steps of the structured engine: the resident kernel
-// where its vectors fit in shared memory, else (and for the lexicographic rule
-// and a priority list, which it does not have) k_iterate_s.
-cudaError_t launch_structured(lp_handle* h, int k_live) {
+// The resident kernel's layout for the next launch (no lexicographic rule and no
+// priority list, which it does not have; vectors that fit in shared memory).
+bool resident_fits(const lp_handle* h, int k_live, ResidentPlan* rp) {
+    return !h->p.lex && !h->p.prio &&
+           resident_plan(h->m, h->n, h->ld, h->r_ctas, k_live, h->opt.graph_iters + 1, h->smem_optin, rp);
+}
+
+// Up to graph_iters + 1 of its steps (one more than graph_iters: the first step
+// after an entry only prices and runs the ratio test, so a reinversion period
+// fits one launch).
+cudaError_t launch_resident(lp_handle* h, const ResidentPlan& rp) {
     const int iters = h->opt.graph_iters + 1;
+    const unsigned seq0 = h->r_seq;
+    h->r_seq += resident_meetings(iters);
+    return launch_iterate_r(h->ds, rp, iters, h->r_meet, seq0, h->stream);
+}
+
+// The structured engine's next launch: the resident kernel, else k_iterate_s.
+cudaError_t launch_structured(lp_handle* h, int k_live) {
     ResidentPlan rp;
-    if (!h->p.lex && !h->p.prio &&
-        resident_plan(h->m, h->n, h->ld, h->r_ctas, k_live, iters, h->smem_optin, &rp)) {
-        const unsigned seq0 = h->r_seq;
-        h->r_seq += resident_meetings(iters);
-        return launch_iterate_r(h->ds, rp, iters, h->r_meet, seq0, h->stream);
-    }
-    return launch_iterate_s(h->ds, h->persist_blocks, iters, h->stream);
+    if (resident_fits(h, k_live, &rp)) return launch_resident(h, rp);
+    return launch_iterate_s(h->ds, h->persist_blocks, h->opt.graph_iters + 1, h->stream);
 }
 
 int reset_state(lp_handle* h) {
@@ -1173,30 +1182,47 @@ int lp_solve(lp_handle* h, lp_result* out) {
         if (h->warm_repair_max < 0) {
             TRY(reinvert(h, 1, false));
         } else {
-            int rc = reinvert(h, 0, false);
+            ResidentPlan rp;
+            const bool resident = h->structured && resident_fits(h, 0, &rp);
+            int rc = reinvert(h, 0, false, resident);
             bool ok = rc == LP_OK;
             if (rc != LP_OK && rc != LP_ERR_SINGULAR) return rc;
             if (ok) {
-                // repair pivots in batches (a captured graph of kRepairBatch
-                // steps), the outcome read once per batch
                 TRY(read_ctrl(h));
                 const int it0 = h->h_ctrl->it;
                 const int limit = it0 + h->warm_repair_max;
                 launch_repair_begin(h->ds, 1e-9 * h->p.b_scale, limit, h->stream);
                 h->launches += 1;
-                if (!h->rgraph) TRY(capture_repair_graph(h));
+                // in the resident kernel where it runs (which goes on with the method
+                // once the start is feasible), else in batches of captured steps on the
+                // dense inverse, whose outcome is read once per batch
+                bool on_chip = resident;
+                if (!on_chip && !h->rgraph) TRY(capture_repair_graph(h));
                 for (;;) {
-                    CK(cudaGraphLaunch(h->rgraph, h->stream));
-                    h->launches += 4 * kRepairBatch;
+                    if (on_chip) {
+                        if (!resident_fits(h, h->h_ctrl->k_live, &rp) || launch_resident(h, rp) != cudaSuccess) {
+                            // (the live slots no longer fit, or the launch was refused)
+                            (void)cudaGetLastError();
+                            on_chip = false;
+                            TRY(reinvert(h, 0, true));
+                            if (!h->rgraph) TRY(capture_repair_graph(h));
+                            continue;
+                        }
+                        h->launches += 1;
+                    } else {
+                        CK(cudaGraphLaunch(h->rgraph, h->stream));
+                        h->launches += 4 * kRepairBatch;
+                    }
                     TRY(read_ctrl(h));
                     const Ctrl& C = *h->h_ctrl;
                     if (C.err != kErrNone) return device_err_code(C.err);
                     if (C.repair == 2) break;                       // feasible
                     if (C.repair >= 3) { ok = false; break; }       // no slack can repair, or the cap
-                    if (C.status == kReinvert) TRY(reinvert(h, 0, true));
+                    if (C.status == kReinvert) TRY(reinvert(h, 0, true, on_chip));
                     else if (C.status != kRunning) break;
                 }
-                warm_repairs = h->h_ctrl->it - it0;
+                const Ctrl& C = *h->h_ctrl;
+                warm_repairs = (on_chip && C.repair >= 2 ? C.repair_end : C.it) - it0;
             }
             if (!ok) {
                 warm_fallback = 1;
@@ -1278,8 +1304,6 @@ int lp_solve(lp_handle* h, lp_result* out) {
             }
             const Ctrl before = C;
             if (h->evc0) CK(cudaEventRecord(h->evc0, h->stream));
-            // one step more than graph_iters: the first step after an entry only
-            // prices and runs the ratio test, so a reinversion period fits one launch
             const cudaError_t e = launch_structured(h, C.k_live);
             if (e == cudaSuccess) {
                 h->launches += 1;
