@@ -78,11 +78,15 @@ __device__ __forceinline__ ulonglong2 ld_acquire_b128(const ulonglong2* p) {
     return v;
 }
 
-// One chunk of the CTA's record under `seq`.  Every CTA has 64 bytes of its own:
-// with the CTAs' chunks side by side (eight per line) the polls of a line hold up its
-// writers, and a meeting of 152 CTAs took 2.3 us instead of 1.0.
-__device__ __forceinline__ void meet_put(ulonglong2* buf, unsigned seq, int chunk, unsigned a, unsigned b, unsigned c) {
-    st_relaxed_b128(buf + ((size_t)(seq & 1) * gridDim.x + blockIdx.x) * kRChunks + chunk,
+// One chunk of the CTA's record under `seq`, into CTA dest's mailbox.  Every CTA has a
+// mailbox of its own, which no other polls, a sender's 16 bytes beside the next
+// sender's: a warp polls 32 senders in four lines, and thread t puts the record into
+// mailbox t.  One record for all, 64 bytes apart and polled by every CTA, held up its writer
+// (17.9 us a pivot against 17.0 at 4096 x 8192 on 152 CTAs, 10.6 against 9.5 at
+// 1024 x 2048); chunks of several CTAs in one line that all poll took 2.3 us a meeting.
+__device__ __forceinline__ void meet_put(ulonglong2* buf, unsigned seq, int dest, int chunk, unsigned a, unsigned b,
+                                         unsigned c) {
+    st_relaxed_b128(buf + (((size_t)(seq & 1) * gridDim.x + dest) * kRChunks + chunk) * gridDim.x + blockIdx.x,
                     ((unsigned long long)b << 32) | a, ((unsigned long long)seq << 32) | c);
 }
 
@@ -91,13 +95,13 @@ __device__ __forceinline__ void meet_put(ulonglong2* buf, unsigned seq, int chun
 // reaches before every CTA has read it.
 template <int C0, int C1>
 __device__ __forceinline__ void meet_get(const ulonglong2* buf, unsigned seq, int c, unsigned* w, volatile int* fail) {
-    const ulonglong2* p = buf + ((size_t)(seq & 1) * gridDim.x + c) * kRChunks;
+    const ulonglong2* p = buf + ((size_t)(seq & 1) * gridDim.x + blockIdx.x) * kRChunks * gridDim.x + c;
     unsigned spins = 0;
     for (;;) {
         ulonglong2 v[C1 - C0];
         bool ok = true;
 #pragma unroll
-        for (int e = C0; e < C1; ++e) v[e - C0] = ld_acquire_b128(p + e);
+        for (int e = C0; e < C1; ++e) v[e - C0] = ld_acquire_b128(p + (size_t)e * gridDim.x);
 #pragma unroll
         for (int e = C0; e < C1; ++e) {
             ok &= (unsigned)(v[e - C0].y >> 32) == seq;
@@ -219,12 +223,12 @@ __device__ __forceinline__ bool tie_near(long long k, long long kmin, double tol
     return h - hm <= 4 || hm < (1023 - 19) << 20 || __double_as_longlong(tol) > (long long)(1023 - 39) << 52;
 }
 
-// The CTA's ratio-test record (one warp): chunk 0 the smallest ratio and the
+// The CTA's ratio-test record (one warp; into w): chunk 0 the smallest ratio and the
 // best row, chunk 1 its alpha and variable, marked kRMore when more than one row
 // ties; then chunk 2 holds the best row's ratio and the size of the tie set.
 // A lone smallest ratio with no other near it needs no threshold.
 __device__ __forceinline__ void ratio_record(const Params& P, int owned, bool bland, const double* ral,
-                                             const double* rb, const int* rvar, ulonglong2* buf, unsigned seq) {
+                                             const double* rb, const int* rvar, unsigned* w) {
     const int lane = threadIdx.x & 31;
     const int G = gridDim.x;
     const long long kpiv = dkey(P.tol_piv), kbig = dkey(DBL_MAX);
@@ -246,10 +250,10 @@ __device__ __forceinline__ void ratio_record(const Params& P, int owned, bool bl
         }
         if (lane == win) {
             const bool none = kmin == kbig, more = cnt > 1;
-            meet_put(buf, seq, 0, ll_lo(kmin), ll_hi(kmin), (unsigned)(none ? -1 : (int)blockIdx.x + G * lane));
             const long long a = __double_as_longlong(al), t = __double_as_longlong(th);
-            meet_put(buf, seq, 1, ll_lo(a), ll_hi(a), none ? 0u : (unsigned)var | (more ? kRMore : 0u));
-            if (more) meet_put(buf, seq, 2, ll_lo(t), ll_hi(t), (unsigned)cnt);
+            w[0] = ll_lo(kmin); w[1] = ll_hi(kmin); w[2] = (unsigned)(none ? -1 : (int)blockIdx.x + G * lane);
+            w[3] = ll_lo(a); w[4] = ll_hi(a); w[5] = none ? 0u : (unsigned)var | (more ? kRMore : 0u);
+            w[6] = ll_lo(t); w[7] = ll_hi(t); w[8] = (unsigned)cnt;
         }
         return;
     }
@@ -259,9 +263,9 @@ __device__ __forceinline__ void ratio_record(const Params& P, int owned, bool bl
     if (lane < 3) {
         const bool more = o.cnt > 1 || dkey(o.th) != o.tmin;
         const long long v = lane == 0 ? o.tmin : __double_as_longlong(lane == 1 ? o.a : o.th);
-        if (lane < 2 || more)
-            meet_put(buf, seq, lane, ll_lo(v), ll_hi(v),
-                     lane == 0 ? (unsigned)o.row : lane == 1 ? (unsigned)o.var | (more ? kRMore : 0u) : (unsigned)o.cnt);
+        w[3 * lane] = ll_lo(v);
+        w[3 * lane + 1] = ll_hi(v);
+        w[3 * lane + 2] = lane == 0 ? (unsigned)o.row : lane == 1 ? (unsigned)o.var | (more ? kRMore : 0u) : (unsigned)o.cnt;
     }
 }
 
@@ -303,7 +307,8 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
     __shared__ PricePatch ppat;
     __shared__ double rinv_sh, cq_sh, thr_sh, dpart[2], cd[kRCand];
     __shared__ int screen_sh;
-    __shared__ unsigned pub[2 * kRList];
+    __shared__ unsigned pub[2 * kRList], rpub[9];
+    __shared__ Cand cpub;
     __shared__ int rep_sh, rep_code, rep_end, rep_row;  // warm-start repair: running, outcome
     __shared__ double rep_val;
     __shared__ int bL, bcnt, bov, nrow, scan_sh;  // the CTA's PRICE record; rows taken by the update; scan
@@ -370,8 +375,8 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
     auto meet = [&] {
         __syncthreads();
         ++seq;
-        if (tid == 0) meet_put(xbuf, seq, 0, 0, 0, 0);
         if (tid < G) {
+            meet_put(xbuf, seq, tid, 0, 0, 0, 0);
             unsigned w[3];
             meet_get<0, 1>(xbuf, seq, tid, w, &fail);
         }
@@ -636,15 +641,18 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
                 if (lane == 0) __threadfence();  // the updated rows, before the record
                 __syncwarp();
                 if (lane == max(win, 0)) {
-                    meet_put(xbuf, seq, 0, ll_lo(wm), ll_hi(wm), (unsigned)(win < 0 ? -1 : pi));
-                    meet_put(xbuf, seq, 1, 0, 0, (unsigned)var);
+                    rpub[0] = ll_lo(wm); rpub[1] = ll_hi(wm); rpub[2] = (unsigned)(win < 0 ? -1 : pi);
+                    rpub[5] = (unsigned)var;
                 }
             }
             if (warp < nwu) {
+                asm volatile("bar.sync 1, %0;\n" ::"r"(32 * nwu) : "memory");
                 unsigned w[kRWords];
                 long long kb = kbig;
                 int pi = INT_MAX, var = 0;
                 if (tid < G) {
+                    meet_put(xbuf, seq, tid, 0, rpub[0], rpub[1], rpub[2]);
+                    meet_put(xbuf, seq, tid, 1, 0, 0, rpub[5]);
                     meet_get<0, 2>(xbuf, seq, tid, w, &fail);
                     kb = words_ll(w[0], w[1]);
                     pi = (int)w[2];
@@ -802,16 +810,15 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
                     offer(hi, j);
                 }
                 asm volatile("bar.sync 1, %0;\n" ::"n"(32 * kRPrice) : "memory");
-                if (warp == 0) {
+                if (tid < G) {
                     // chunk 0 says all when at most one column is listed
                     const int cnt = min(bcnt, kRList);
-                    if (lane == 0) {
-                        meet_put(xbuf, seq, 0, (unsigned)bL, cnt ? pub[0] : (unsigned)INT_MIN,
-                                 (cnt ? pub[1] : 0u) | (cnt > 1 ? kRMore : 0u));
-                    } else if (cnt > 1 && lane < 4) {
-                        if (lane == 1) meet_put(xbuf, seq, 1, (unsigned)cnt, pub[2], pub[3]);
-                        else if (lane == 2) meet_put(xbuf, seq, 2, (unsigned)bov, pub[4], pub[5]);
-                        else meet_put(xbuf, seq, 3, 0, pub[6], pub[7]);
+                    meet_put(xbuf, seq, tid, 0, (unsigned)bL, cnt ? pub[0] : (unsigned)INT_MIN,
+                             (cnt ? pub[1] : 0u) | (cnt > 1 ? kRMore : 0u));
+                    if (cnt > 1) {
+                        meet_put(xbuf, seq, tid, 1, (unsigned)cnt, pub[2], pub[3]);
+                        meet_put(xbuf, seq, tid, 2, (unsigned)bov, pub[4], pub[5]);
+                        meet_put(xbuf, seq, tid, 3, 0, pub[6], pub[7]);
                     }
                 }
                 if (warp < nwu) {
@@ -948,13 +955,16 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
                 cand_init(cand);
                 if (lane < kRWarps) cand = wcand[lane];
                 cand = cand_warp_reduce(cand);
-                if (lane == 0) meet_put(xbuf, seq, 0, ll_lo(cand.d_all), ll_hi(cand.d_all), (unsigned)cand.j_all);
-                if (lane == 1) meet_put(xbuf, seq, 1, ll_lo(cand.d_nt), ll_hi(cand.d_nt), (unsigned)cand.j_nt);
-                if (lane == 2) meet_put(xbuf, seq, 2, ll_lo(cand.d_min), ll_hi(cand.d_min), (unsigned)cand.j_min);
+                if (lane == 0) cpub = cand;
             }
-            __syncthreads();  // (wcand is written again)
+            __syncthreads();  // (and wcand is written again)
             if (warp < nwu) {
                 unsigned w[kRWords];
+                if (tid < G) {
+                    meet_put(xbuf, seq, tid, 0, ll_lo(cpub.d_all), ll_hi(cpub.d_all), (unsigned)cpub.j_all);
+                    meet_put(xbuf, seq, tid, 1, ll_lo(cpub.d_nt), ll_hi(cpub.d_nt), (unsigned)cpub.j_nt);
+                    meet_put(xbuf, seq, tid, 2, ll_lo(cpub.d_min), ll_hi(cpub.d_min), (unsigned)cpub.j_min);
+                }
                 cand_init(cand);
                 if (tid < G) {
                     meet_get<0, 3>(xbuf, seq, tid, w, &fail);
@@ -1072,13 +1082,11 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
         // ---- the CTA's ratio-test record
         ++seq;
         if (warp == 0) {
-            ratio_record(P, owned, bland, al, bb, rvar, xbuf, seq);
+            ratio_record(P, owned, bland, al, bb, rvar, rpub);
         } else if (tid == kRThreads - 32 && !dq_known) {
             S.dq = qn < n ? cq_sh - (dpart[0] + dpart[1]) : -ycur[rs[qn - n]];
         }
         if (warp < nwu) {
-            // no polling before this CTA's own record is out: the polls of 152 CTAs
-            // would only delay the records
             asm volatile("bar.sync 1, %0;\n" ::"r"(32 * nwu) : "memory");
             unsigned w[kRWords];
             long long tmin = kbig;
@@ -1086,6 +1094,9 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
             int var = 0, row = -1;
             bool more = false;
             if (tid < G) {
+                meet_put(xbuf, seq, tid, 0, rpub[0], rpub[1], rpub[2]);
+                meet_put(xbuf, seq, tid, 1, rpub[3], rpub[4], rpub[5]);
+                if (rpub[5] & kRMore) meet_put(xbuf, seq, tid, 2, rpub[6], rpub[7], rpub[8]);
                 meet_get<0, 2>(xbuf, seq, tid, w, &fail);
                 tmin = words_ll(w[0], w[1]);
                 row = (int)w[2];
@@ -1233,7 +1244,7 @@ int resident_ctas(int sms, int m, int n) {
     return std::max(1, std::min(std::min(g, std::max(m, n)), std::min(kRMaxCtas, sms)));
 }
 
-size_t resident_meet_bytes(int ctas) { return sizeof(ulonglong2) * 2 * kRChunks * (size_t)ctas; }
+size_t resident_meet_bytes(int ctas) { return sizeof(ulonglong2) * 2 * kRChunks * (size_t)ctas * ctas; }
 
 bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t smem_optin, ResidentPlan* out) {
     constexpr size_t kStatic = 4096;  // static shared memory of the kernel, rounded up
