@@ -495,58 +495,119 @@ __global__ void k_refine_extract(DevState s, int k, int from_struct, int k_live,
     }
 }
 
-// kMode 0: R[i][c] = [i == c] - sum_l B11[i][l] Y0[l][c], and the sum of |R|
-//          over the tile's columns (in column order) per row into the partials;
-// kMode 1: Y1[i][c] = Y0[i][c] + sum_l Y0[i][l] R[l][c], into rv_W.
+// The two products in FP64.
+// kMode 0: R[i][c] = [i == c] - sum_l B11[i][l] Y0[l][c] from the extracted operands, and
+//          the sum of |R| over the tile's columns (in column order) per row into the partials;
+// kMode 1: the same, with both operands gathered from A and the live columns of B^-1
+//          here (no k_refine_extract before it); the first row of tiles leaves Y0 for kMode 2;
+// kMode 2: Y1[i][c] = Y0[i][c] + sum_l Y0[i][l] R[l][c], into rv_W; the first column of
+//          tiles sums the partials (in tile order) into ||R||_inf, as k_refine_finish_residual.
 // Each output is one fused multiply-add chain in increasing l, so the result
-// does not depend on the launch shape.  kRT x kRT tiles keep the SMs' shares
-// within one small tile of each other at k of a few hundred.
-constexpr int kRT = 8;
+// does not depend on the launch shape.  kRT x kRT tiles of two warps keep the SMs' shares
+// within one small tile of each other: an FP64 instruction holds its SM's pipe for 16
+// cycles, and at k = 64 each of the 64 tiles has an SM to itself.  The next kRC columns
+// are on their way while a chunk is multiplied.
+// The FP64 products up to this k, the sliced ones beyond: two launches instead of nine,
+// but k^3 FP64 operations.  Both products, us at k = 32, 64, 128, 160, 192: 13, 17, 23, 33, 44
+// here, 31, 32, 35, 38, 38 sliced.
+constexpr int kRefineFp64 = 160;
+constexpr int kRT = 8, kRC = 64;
 template <int kMode>
-__global__ void __launch_bounds__(kRT * kRT) k_refine_gemm(DevState s, int k) {
+__global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int k_live, int par) {
+    pdl_enter();
     if (s.ctrl->err != kErrNone) return;
+    __shared__ double xs[kRT][kRC + 1], zs[kRC][kRT];
+    constexpr int kU = kRC / kRT;  // a thread's elements of each operand's chunk
     const size_t kk = (size_t)k * k;
-    const double* B11 = s.rv_M;
-    const double* Y0 = s.rv_M + kk;
+    double* Y0 = s.rv_M + kk;
     double* R = s.rv_M + 2 * kk;
-    const int tx = threadIdx.x % kRT, ty = threadIdx.x / kRT;
-    const int i = blockIdx.y * kRT + ty, c = blockIdx.x * kRT + tx;
+    const int tid = threadIdx.x, tx = tid % kRT, ty = tid / kRT;
+    const int i0 = blockIdx.y * kRT, c0 = blockIdx.x * kRT;
+    const int i = i0 + ty, c = c0 + tx;
     const bool in = i < k && c < k;
-    double acc = 0.0;
-    if (in) {
-        if (kMode == 0) {
-            const double* x = B11 + i;  // B11[i][l] at l*k + i
-            const double* z = Y0 + c;   // Y0[l][c] at l*k + c
-#pragma unroll 8
-            for (int l = 0; l < k; ++l) acc = fma(x[(size_t)l * k], z[(size_t)l * k], acc);
-        } else {
-            const double* x = Y0 + (size_t)i * k;  // Y0[i][l]
-            const double* z = R + c;               // R[l][c] at l*k + c
-#pragma unroll 8
-            for (int l = 0; l < k; ++l) acc = fma(x[l], z[(size_t)l * k], acc);
+    const int nt = gridDim.x;
+    // the row (of B11) and the column (of Y0) whose elements this thread stages; the
+    // indexes of l are in shared memory before the first gather (an index loaded beside its
+    // element stalls the thread once per element: 15 us a chunk instead of 3)
+    __shared__ int jl[kMode == 1 ? kRefineFp64 : 1], pl[kMode == 1 ? kRefineFp64 : 1];
+    int xrow = 0, zcol = -1;
+    if (kMode == 1) {
+        for (int l = tid; l < k; l += kRT * kRT) {
+            jl[l] = s.rv_J[l];
+            pl[l] = s.rv_struct_pos[l];
         }
-    }
-    if (kMode == 0) {
-        __shared__ double rabs[kRT][kRT];
-        double v = 0.0;
-        if (in) {
-            v = (i == c ? 1.0 : 0.0) - acc;
-            R[(size_t)i * k + c] = v;
+        if (i0 + tx < k) xrow = s.rv_rows[i0 + tx];
+        if (c < k) {
+            const int sl = s.row_slot[(size_t)par * s.p.m + s.rv_rows[c]];
+            if (sl >= 0 && sl < k_live) zcol = sl;
         }
-        rabs[ty][tx] = fabs(v);
         __syncthreads();
-        if (tx == 0 && i < k) {
-            double t = 0.0;
+    }
+    double xv[kU], zv[kU];
+    auto fetch = [&](int l0) {
 #pragma unroll
-            for (int u = 0; u < kRT; ++u) t += rabs[ty][u];
-            s.rv_W[kk + (size_t)i * gridDim.x + blockIdx.x] = t;
+        for (int u = 0; u < kU; ++u) {
+            // B11 by columns (element ty + 8 u of a column's rows), Y0 by rows
+            const int l = l0 + ty + kRT * u;
+            xv[u] = zv[u] = 0.0;
+            if (l >= k) continue;
+            if (kMode == 1) {
+                if (i0 + tx < k) xv[u] = s.A_cm[(size_t)jl[l] * s.p.ld + xrow];
+                if (zcol >= 0) zv[u] = s.bp[(size_t)pl[l] * s.p.ld + zcol];
+            } else {
+                if (kMode == 0) {
+                    if (i0 + tx < k) xv[u] = s.rv_M[(size_t)l * k + i0 + tx];
+                    if (c < k) zv[u] = Y0[(size_t)l * k + c];
+                } else {
+                    if (i0 + tx < k) xv[u] = Y0[(size_t)(i0 + tx) * k + l];
+                    if (c < k) zv[u] = R[(size_t)l * k + c];
+                }
+            }
         }
-    } else if (in) {
-        s.rv_W[(size_t)i * k + c] = Y0[(size_t)i * k + c] + acc;
+    };
+    fetch(0);
+    double acc = 0.0;
+    for (int l0 = 0; l0 < k; l0 += kRC) {
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int l = ty + kRT * u;
+            xs[tx][l] = xv[u];
+            zs[l][tx] = zv[u];
+            if (kMode == 1 && blockIdx.y == 0 && l0 + l < k && c < k) Y0[(size_t)(l0 + l) * k + c] = zv[u];
+        }
+        __syncthreads();
+        fetch(l0 + kRC);
+        const int w = min(kRC, k - l0);
+#pragma unroll 16
+        for (int l = 0; l < w; ++l) acc = fma(xs[ty][l], zs[l][tx], acc);
+        __syncthreads();
+    }
+    if (kMode == 2) {
+        if (in) s.rv_W[(size_t)i * k + c] = Y0[(size_t)i * k + c] + acc;
+        if (blockIdx.x == 0 && tx == 0 && i < k) {
+            double t = 0.0;
+            for (int u = 0; u < nt; ++u) t += s.rv_W[kk + (size_t)i * nt + u];
+            atomicMax(reinterpret_cast<unsigned long long*>(&s.ctrl->refine_res),
+                      (unsigned long long)__double_as_longlong(t >= 0.0 ? t : DBL_MAX));
+        }
+        return;
+    }
+    double v = 0.0;
+    if (in) {
+        v = (i == c ? 1.0 : 0.0) - acc;
+        R[(size_t)i * k + c] = v;
+    }
+    zs[ty][tx] = fabs(v);
+    __syncthreads();
+    if (tx == 0 && i < k) {
+        double t = 0.0;
+#pragma unroll
+        for (int u = 0; u < kRT; ++u) t += zs[ty][u];
+        s.rv_W[kk + (size_t)i * nt + blockIdx.x] = t;
     }
 }
 
-// Tensor-core form of the two products (reinvert_tc, k <= 1024): the exact
+// Tensor-core form of the two products (reinvert_tc, kRefineFp64 < k <= 1024): the exact
 // 7-bit-sliced products of ozaki.cu give P = -(B11 Y0) into R's place and
 // P = Y0 R into rv_W; these kernels finish them.
 // R = I - B11 Y0 = I + P in place, and ||R||_inf into ctrl->refine_res (reset
@@ -584,29 +645,6 @@ __global__ void k_refine_add(DevState s, int k) {
     const double* Y0 = s.rv_M + kk;
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < kk; e += (size_t)gridDim.x * blockDim.x)
         s.rv_W[e] = Y0[e] + s.rv_W[e];
-}
-
-// ||R||_inf from the partial row sums (each row summed in tile order) into
-// ctrl->refine_res; a NaN row counts as infinite.
-__global__ void __launch_bounds__(1024) k_refine_norm(DevState s, int k, int ntc) {
-    __shared__ double wmax[32];
-    const double* part = s.rv_W + (size_t)k * k;
-    double mx = 0.0;
-    if (s.ctrl->err == kErrNone)
-        for (int a = threadIdx.x; a < k; a += blockDim.x) {
-            double r = 0.0;
-            for (int t = 0; t < ntc; ++t) r += part[(size_t)a * ntc + t];
-            if (!(r >= 0.0)) r = DBL_MAX;  // NaN
-            mx = fmax(mx, r);
-        }
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double m = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, wmax[w]);
-        s.ctrl->refine_res = s.ctrl->err == kErrNone ? m : DBL_MAX;
-    }
 }
 
 // pinv[pivrow[t]] = t (stored over rv_rowdone, no longer needed)
@@ -896,41 +934,34 @@ void launch_reinv_gj(const DevState& s, int k, const Geometry& g, cudaStream_t s
 
 bool refine_fits(int k, int m) { return k > 0 && 3 * (size_t)k * k <= (size_t)m * m; }
 
-static bool refine_on_tc(const DevState& s, int k) { return s.p.reinvert_tc && s.oz_xs && oz_fits(k); }
-
-// Returns the number of kernels launched.
-int launch_refine_residual(const DevState& s, int k, int from_struct, int k_live, int par, cudaStream_t st) {
+// Y1 into rv_W and ||R||_inf into the control block.  Returns the number of
+// kernels launched.
+int launch_refine(const DevState& s, int k, int from_struct, int k_live, int par, cudaStream_t st) {
     const size_t kk = (size_t)k * k;
+    const int nt = (k + kRT - 1) / kRT;
+    const dim3 tiles(nt, nt), tile(kRT * kRT);
+    if (from_struct && k <= kRefineFp64) {
+        launch_k(k_refine_fp64<1>, tiles, tile, 0, st, true, s, k, k_live, par);
+        launch_k(k_refine_fp64<2>, tiles, tile, 0, st, true, s, k, k_live, par);
+        return 2;
+    }
     int blocks = (int)((kk + 255) / 256);
     if (blocks > 4096) blocks = 4096;
     launch_k(k_refine_extract, dim3(blocks), dim3(256), 0, st, true, s, k, from_struct, k_live, par);
-    if (refine_on_tc(s, k) &&
+    if (k > kRefineFp64 && s.p.reinvert_tc && s.oz_xs && oz_fits(k) &&
         oz_refine_residual_product(s.rv_M, s.rv_M + kk, k, s.rv_M + 2 * kk, s.oz_xs, s.oz_ys, s.oz_ex, s.oz_ey,
                                    &s.ctrl->err, st) == cudaSuccess) {
         launch_k(k_refine_finish_residual, dim3((k + 7) / 8), dim3(256), 0, st, true, s, k);
-        return 5;
+        if (oz_refine_update_product(s.rv_M + kk, s.rv_M + 2 * kk, k, s.rv_W, s.oz_xs, s.oz_ys, s.oz_ex, s.oz_ey,
+                                     &s.ctrl->err, st) == cudaSuccess) {
+            launch_k(k_refine_add, dim3(blocks), dim3(256), 0, st, true, s, k);
+            return 9;
+        }
     }
     (void)cudaGetLastError();
-    const int nt = (k + kRT - 1) / kRT;
-    k_refine_gemm<0><<<dim3(nt, nt), kRT * kRT, 0, st>>>(s, k);
-    k_refine_norm<<<1, 1024, 0, st>>>(s, k, nt);
+    launch_k(k_refine_fp64<0>, tiles, tile, 0, st, true, s, k, k_live, par);
+    launch_k(k_refine_fp64<2>, tiles, tile, 0, st, true, s, k, k_live, par);
     return 3;
-}
-
-int launch_refine_apply(const DevState& s, int k, cudaStream_t st) {
-    const size_t kk = (size_t)k * k;
-    if (refine_on_tc(s, k) &&
-        oz_refine_update_product(s.rv_M + kk, s.rv_M + 2 * kk, k, s.rv_W, s.oz_xs, s.oz_ys, s.oz_ex, s.oz_ey,
-                                 &s.ctrl->err, st) == cudaSuccess) {
-        int blocks = (int)((kk + 255) / 256);
-        if (blocks > 4096) blocks = 4096;
-        launch_k(k_refine_add, dim3(blocks), dim3(256), 0, st, true, s, k);
-        return 4;
-    }
-    (void)cudaGetLastError();
-    const int nt = (k + kRT - 1) / kRT;
-    k_refine_gemm<1><<<dim3(nt, nt), kRT * kRT, 0, st>>>(s, k);
-    return 1;
 }
 
 // Returns 1 when the slack-row product ran on the tensor cores.  dense_rows:

@@ -348,8 +348,7 @@ cudaError_t oz_refine_residual_product(const double* B11_cm, const double* Y0, i
                                        int32_t* err, cudaStream_t st);
 cudaError_t oz_refine_update_product(const double* Y0, const double* R, int k, double* P, __nv_bfloat16* xs,
                                      __nv_bfloat16* ys, int32_t* ex, int32_t* ey, int32_t* err, cudaStream_t st);
-int launch_refine_residual(const DevState& s, int k, int from_struct, int k_live, int par, cudaStream_t st);
-int launch_refine_apply(const DevState& s, int k, cudaStream_t st);
+int launch_refine(const DevState& s, int k, int from_struct, int k_live, int par, cudaStream_t st);
 // refine_tol >= 0: the rebuild came from a refinement, accepted when its residual is <= refine_tol
 void launch_reinv_finish(const DevState& s, int k, const Geometry& g, cudaStream_t st, int check_feasible,
                          double refine_tol);

@@ -425,9 +425,7 @@ int reinvert_queue(lp_handle* h, int check_feasible, bool refine, bool to_struct
     CK(cudaEventRecord(h->erg, h->stream));
     if (q->try_refine) {
         const bool from_struct = h->structured && h->s_ready;
-        h->launches += launch_refine_residual(h->ds, k, from_struct ? 1 : 0, h->h_ctrl->k_live, h->h_ctrl->map_par,
-                                              h->stream);
-        h->launches += launch_refine_apply(h->ds, k, h->stream);
+        h->launches += launch_refine(h->ds, k, from_struct ? 1 : 0, h->h_ctrl->k_live, h->h_ctrl->map_par, h->stream);
     } else {
         launch_reinv_gj(h->ds, k, h->geo, h->stream);
         h->launches += reinv_gj_launches(k);
