@@ -502,16 +502,23 @@ __global__ void k_refine_extract(DevState s, int k, int from_struct, int k_live,
 //          here (no k_refine_extract before it); the first row of tiles leaves Y0 for kMode 2;
 // kMode 2: Y1[i][c] = Y0[i][c] + sum_l Y0[i][l] R[l][c], into rv_W; the first column of
 //          tiles sums the partials (in tile order) into ||R||_inf, as k_refine_finish_residual.
-// Each output is one fused multiply-add chain in increasing l, so the result
-// does not depend on the launch shape.  kRT x kRT tiles of two warps keep the SMs' shares
-// within one small tile of each other: an FP64 instruction holds its SM's pipe for 16
-// cycles, and at k = 64 each of the 64 tiles has an SM to itself.  The next kRC columns
-// are on their way while a chunk is multiplied.
-// The FP64 products up to this k, the sliced ones beyond: two launches instead of nine,
-// but k^3 FP64 operations.  Both products, us at k = 32, 64, 128, 160, 192: 13, 17, 23, 33, 44
-// here, 31, 32, 35, 38, 38 sliced.
-constexpr int kRefineFp64 = 160;
+// Each output is one chain in increasing l, so the result does not depend on the launch
+// shape.  R's sum runs beside a bias, which holds every addend to a multiple of
+// 2^-32 as long as the sum stays below 2^19; what that cuts off each product (exact: a
+// fused multiply-add of it) goes into a second sum.  So R has no rounding error to
+// speak of, and Y1 little more than that of its last addition: with these sums at every k, x
+// of 200 x 300 and 260 x 500 LPs came out at 3e-14 and 4e-14 of the exact solution (geometric
+// means), 1.5e-13 and 2.7e-13 with plain sums, 1.1e-13 and 1.8e-13 with sliced products.
+// kRT x kRT tiles of two warps: an FP64 instruction holds its SM's pipe for 16
+// cycles, and at k = 64 each of the 64 tiles has an SM to itself.  The next kRC columns are
+// on their way while a chunk is multiplied.
+// kRefineFp64: these products up to this k, the sliced ones beyond (two launches instead of
+// nine, but k^3 FP64 operations, four per element of R's sums).  Both products, us at
+// k = 32, 64, 96, 128: 15, 22, 30-56, 35-72 here (tiles then share SMs),
+// 31, 32, 36, 36 sliced.
+constexpr int kRefineFp64 = 64;
 constexpr int kRT = 8, kRC = 64;
+constexpr double kRBias = 1.5 * (1 << 20);
 template <int kMode>
 __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int k_live, int par) {
     pdl_enter();
@@ -528,7 +535,7 @@ __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int
     const int nt = gridDim.x;
     // the row (of B11) and the column (of Y0) whose elements this thread stages; the
     // indexes of l are in shared memory before the first gather (an index loaded beside its
-    // element stalls the thread once per element: 15 us a chunk instead of 3)
+    // element stalls the thread once per element)
     __shared__ int jl[kMode == 1 ? kRefineFp64 : 1], pl[kMode == 1 ? kRefineFp64 : 1];
     int xrow = 0, zcol = -1;
     if (kMode == 1) {
@@ -566,7 +573,7 @@ __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int
         }
     };
     fetch(0);
-    double acc = 0.0;
+    double acc = kMode == 2 ? 0.0 : kRBias, lo = 0.0;
     for (int l0 = 0; l0 < k; l0 += kRC) {
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
@@ -577,9 +584,14 @@ __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int
         }
         __syncthreads();
         fetch(l0 + kRC);
-        const int w = min(kRC, k - l0);
-#pragma unroll 16
-        for (int l = 0; l < w; ++l) acc = fma(xs[ty][l], zs[l][tx], acc);
+        for (int l1 = 0; l1 < k - l0 && l1 < kRC; l1 += 16)  // (zeros past k)
+#pragma unroll
+            for (int l = l1; l < l1 + 16; ++l) {
+                const double x = xs[ty][l], z = zs[l][tx];
+                const double t = fma(x, z, acc);
+                if (kMode != 2) lo += fma(x, z, acc - t);
+                acc = t;
+            }
         __syncthreads();
     }
     if (kMode == 2) {
@@ -594,7 +606,7 @@ __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int
     }
     double v = 0.0;
     if (in) {
-        v = (i == c ? 1.0 : 0.0) - acc;
+        v = ((i == c ? 1.0 : 0.0) - (acc - kRBias)) - lo;
         R[(size_t)i * k + c] = v;
     }
     zs[ty][tx] = fabs(v);
