@@ -21,6 +21,7 @@
 //       B11^-1[b][p_t] = M[p_b][t].
 #include "lpgb_internal.cuh"
 
+#include <algorithm>
 #include <cooperative_groups.h>
 
 #include <cfloat>
@@ -461,7 +462,7 @@ __global__ void __launch_bounds__(kTrailThreads) k_gj_trail(DevState s, int k, i
 // elimination.  A larger residual (or a NaN) falls back to Gauss-Jordan.
 //
 // Scratch: B11 (column-major, as k_gather writes it), Y0 and R = I - B11 Y0
-// (row-major) in rv_M, which needs 3 k^2 <= m^2; per-tile partial row sums of
+// (row-major) in rv_M (refine_fits); per-tile partial row sums of
 // |R| after the first k^2 entries of rv_W; Y1 into rv_W, where the
 // elimination leaves B11^-1.
 
@@ -516,7 +517,8 @@ __global__ void k_refine_extract(DevState s, int k, int from_struct, int k_live,
 // nine, but k^3 FP64 operations, four per element of R's sums).  Both products, us at
 // k = 32, 64, 96, 128: 15, 22, 30-56, 35-72 here (tiles then share SMs),
 // 31, 32, 36, 36 sliced.
-constexpr int kRefineFp64 = 64;
+// kRefineDense: where 3 k^2 > m^2, these products up to this k (refine_fits).
+constexpr int kRefineFp64 = 64, kRefineDense = 256;
 constexpr int kRT = 8, kRC = 64;
 constexpr double kRBias = 1.5 * (1 << 20);
 template <int kMode>
@@ -536,7 +538,7 @@ __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int
     // the row (of B11) and the column (of Y0) whose elements this thread stages; the
     // indexes of l are in shared memory before the first gather (an index loaded beside its
     // element stalls the thread once per element)
-    __shared__ int jl[kMode == 1 ? kRefineFp64 : 1], pl[kMode == 1 ? kRefineFp64 : 1];
+    __shared__ int jl[kMode == 1 ? kRefineDense : 1], pl[kMode == 1 ? kRefineDense : 1];
     int xrow = 0, zcol = -1;
     if (kMode == 1) {
         for (int l = tid; l < k; l += kRT * kRT) {
@@ -944,7 +946,21 @@ void launch_reinv_gj(const DevState& s, int k, const Geometry& g, cudaStream_t s
     k_pivinv<<<(k + 255) / 256, 256, 0, st>>>(s, k);
 }
 
-bool refine_fits(int k, int m) { return k > 0 && 3 * (size_t)k * k <= (size_t)m * m; }
+// The refinement's three k x k blocks have room in rv_M where 3 k^2 <= m^2, and up to
+// k = kRefineDense always: a basis that is mostly structural is refined too, with the FP64
+// products, whose error is the smaller one.  Eliminated afresh, as every such k was, a
+// 200 x 300 LP with k about 150 took 370 us a reinversion instead of 96.
+size_t reinv_m_elems(int m) {
+    const size_t k = std::min(m, kRefineDense);
+    return std::max((size_t)m * m, 3 * k * k);
+}
+// B11^-1 and the slack rows are m k elements; the FP64 products keep k ceil(k / 8) partial
+// sums behind B11^-1
+size_t reinv_w_elems(int m) {
+    const size_t k = std::min(m, kRefineDense);
+    return std::max((size_t)m * m, k * k + k * ((k + kRT - 1) / kRT));
+}
+bool refine_fits(int k, int m) { return k > 0 && (k <= kRefineDense || 3 * (size_t)k * k <= (size_t)m * m); }
 
 // Y1 into rv_W and ||R||_inf into the control block.  Returns the number of
 // kernels launched.
@@ -952,7 +968,8 @@ int launch_refine(const DevState& s, int k, int from_struct, int k_live, int par
     const size_t kk = (size_t)k * k;
     const int nt = (k + kRT - 1) / kRT;
     const dim3 tiles(nt, nt), tile(kRT * kRT);
-    if (from_struct && k <= kRefineFp64) {
+    const bool fp64 = k <= kRefineFp64 || 3 * kk > (size_t)s.p.m * s.p.m;
+    if (from_struct && fp64) {
         launch_k(k_refine_fp64<1>, tiles, tile, 0, st, true, s, k, k_live, par);
         launch_k(k_refine_fp64<2>, tiles, tile, 0, st, true, s, k, k_live, par);
         return 2;
@@ -960,7 +977,7 @@ int launch_refine(const DevState& s, int k, int from_struct, int k_live, int par
     int blocks = (int)((kk + 255) / 256);
     if (blocks > 4096) blocks = 4096;
     launch_k(k_refine_extract, dim3(blocks), dim3(256), 0, st, true, s, k, from_struct, k_live, par);
-    if (k > kRefineFp64 && s.p.reinvert_tc && s.oz_xs && oz_fits(k) &&
+    if (!fp64 && s.p.reinvert_tc && s.oz_xs && oz_fits(k) &&
         oz_refine_residual_product(s.rv_M, s.rv_M + kk, k, s.rv_M + 2 * kk, s.oz_xs, s.oz_ys, s.oz_ex, s.oz_ey,
                                    &s.ctrl->err, st) == cudaSuccess) {
         launch_k(k_refine_finish_residual, dim3((k + 7) / 8), dim3(256), 0, st, true, s, k);

@@ -216,14 +216,16 @@ struct DevState {
     int32_t* rv_g_of_row;    // m: row -> index in rv_slack_pos, or -1
     int32_t* rv_J;           // k: structural variable of index b
     double* rv_cJ;           // k: its cost
-    double* rv_W;            // m*m: dense B11^-1 (k x k) then -A[S,J] B11^-1 ((m-k) x k)
+    double* rv_W;            // dense B11^-1 (k x k) then -A[S,J] B11^-1 ((m-k) x k); after B11^-1
+                             // also the FP64 refinement's partial row sums (reinv_w_elems)
     int32_t* rv_pivrow;      // k: pivot row chosen for column t (GJ)
     int32_t* rv_rowdone;     // k: row already used as pivot
     __nv_bfloat16* oz_xs;    // reinvert_tc: 7-bit slices of A[S, J] (8 rows per slack row), or null
     __nv_bfloat16* oz_ys;    // reinvert_tc: slices of B11^-1 (8 rows per column)
     int32_t* oz_ex;          // reinvert_tc: row exponents of A[S, J] (m)
     int32_t* oz_ey;          // reinvert_tc: column exponents of B11^-1 (m)
-    double* rv_M;            // k*k column-major workspace (B11 then its GJ form)
+    double* rv_M;            // k*k column-major workspace (B11 then its GJ form); the
+                             // refinement's B11, Y0 and R, 3 k^2 (reinv_m_elems)
     double* rv_f;            // 2*k published pivot columns
 };
 
@@ -329,6 +331,8 @@ void launch_reinv_classify(const DevState& s, int k_expect, cudaStream_t st);
 void launch_reinv_gj(const DevState& s, int k, const Geometry& g, cudaStream_t st);
 int reinv_gj_launches(int k);
 int launch_reinv_assemble(const DevState& s, int k, const Geometry& g, cudaStream_t st, int from_gj, bool dense_rows);
+size_t reinv_m_elems(int m);  // rv_M and rv_W
+size_t reinv_w_elems(int m);
 bool refine_fits(int k, int m);
 // Case 2 out-of-core blocks of B^-1 (ooc.cu)
 void launch_ooc_update(const DevState& s, const Geometry& g, double* win, int i0, int i1, cudaStream_t st);

@@ -889,8 +889,8 @@ static int create_impl(lp_handle* h, int32_t m, int32_t n, const double* A, cons
     TRY(dalloc(h, &rv_piv, (size_t)m));
     TRY(dalloc(h, &rv_done, (size_t)m));
     TRY(dalloc(h, &rv_slack, (size_t)m));
-    TRY(dalloc(h, &rv_M, (size_t)m * m));
-    TRY(dalloc(h, &s.rv_W, (size_t)m * m));
+    TRY(dalloc(h, &rv_M, reinv_m_elems(m)));
+    TRY(dalloc(h, &s.rv_W, reinv_w_elems(m)));
     TRY(dalloc(h, &s.rv_b_of_pos, (size_t)m));
     TRY(dalloc(h, &s.rv_g_of_row, (size_t)m));
     TRY(dalloc(h, &s.rv_J, (size_t)m));
