@@ -1233,11 +1233,12 @@ ResKernel res_kernel(bool a, bool b) {
 
 // CTAs of a launch.  A CTA's share of the screen, the update and FTRAN falls with
 // the number of CTAs, and the two meetings of a pivot grow with it (one warp polls
-// up to 32 records: 0.6 us; five warps 152 records: 1.2 us and a second reduction).
-// Measured, us per pivot at 16 / 32 / 80 / 152 CTAs: 128 x 256 8.4 / 8.6 / 10.7 / 10.5,
-// 256 x 512 9.6 / 8.6 / 9.3 / 10.4, 701 x 1203 14 / 10.5 / 9.4 / 9.9, 1024 x 2048
-// 17 / 11.9 / 10.7 / 10.5, 2048 x 4096 - / - / 15.7 / 12.7: the best number follows
-// the cube root of m n, with one polling warp wherever that is near.
+// up to 32 records, five warps 152 and a second reduction).
+// Measured, us per pivot at 16 / 32 / 64 / 112 / 152 CTAs: 128 x 256 8.4 / 8.6 / 9.0 /
+// 9.5 / 10.1, 256 x 512 9.3 / 8.3 / 8.5 / 9.0 / 9.8, 512 x 1024 11.2 / 9.6 / 8.8 / 9.1 / 9.7,
+// 701 x 1203 - / 10.1 / 9.0 / 9.1 / 9.8, 1024 x 2048 - / 12.2 / 10.4 / 9.5 / 10.1, 2048 x 4096
+// - / - / - / 12.6 / 11.8: the best number follows the cube root of m n, with one polling
+// warp wherever that is near.
 int resident_ctas(int sms, int m, int n) {
     int g = (int)std::lround(0.85 * std::cbrt((double)m * n));
     if (g < 56) g = std::min(std::max(g, 16), 32);
