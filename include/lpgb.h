@@ -364,7 +364,8 @@ int lp_get_trace(const lp_handle* h, int32_t* q, int32_t* r, double* theta,
  *
  * All pointers are DEVICE pointers owned by the caller:
  *  A_colmajor  n columns of lda doubles (column j at A_colmajor + j*lda),
- *              16-byte aligned; only the first m entries of a column are read
+ *              16-byte aligned; only the first m entries of a column are read,
+ *              and of those the rows with y_i = 0 may be left out (A is finite)
  *  lda         >= m and even
  *  c (n), y (m), pos (n+m: pos[j] >= 0 marks a basic variable)
  *  q_out (1 int32), dq_out (1 double)
@@ -431,7 +432,7 @@ typedef struct lp_batch_result {
     int32_t failed;          /* LPs whose reinversion met a singular basis */
     int64_t iterations;      /* pivots summed over the batch */
     double seconds;          /* device time of the solve (CUDA events) */
-    double fp64_flops;       /* algorithmic FP64 flops: FTRAN + update + re-pricing */
+    double fp64_flops;       /* FP64 flops of the dense method: FTRAN + update + re-pricing (the kernel leaves out exact zeros) */
 } lp_batch_result;
 
 /*

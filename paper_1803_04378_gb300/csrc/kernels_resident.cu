@@ -16,9 +16,9 @@
 // reinversion reads the whole.  At 4096 x 8192, G = 152 and k = 344 that is
 // 74 KB of A and 74 KB of B^-1 per CTA.
 //
-// Meeting.  The two grid barriers of a pivot carry the CTAs' records: a CTA
-// publishes 48 bytes, each 16-byte chunk stamped with the sequence number of the
-// meeting, and thread c of every CTA polls the chunks of CTA c.  Reading every
+// Meeting.  The two grid barriers of a pivot carry the CTAs' records: thread c of a
+// CTA puts the record into CTA c's mailbox, each 16-byte chunk stamped with the sequence
+// number of the meeting, and then polls its own mailbox for CTA c's.  Reading every
 // CTA's record is the barrier, so a meeting costs one store and one load round
 // trip instead of an atomic, a poll and the records' own loads.
 //
@@ -36,13 +36,13 @@
 // The rank-1 update (warps kRPrice .., then the pricing warps that do not poll)
 // runs under PRICE and its meeting, since only FTRAN needs it.
 //
-// What bounds it: latency.  A pivot is a chain of two meetings (1.1 us each), two L2
+// What bounds it: latency.  A pivot is a chain of two meetings, two L2
 // round trips (pivot row, entering column; 0.6 us each), seven block barriers and
-// the reductions between them; of 17.7 us at 4096 x 8192 the FP64 pipe needs 2.6 us for
+// the reductions between them; of 17.0 us at 4096 x 8192 the FP64 pipe needs 2.6 us for
 // FTRAN, and 2.5 us for the update that PRICE hides.  Against k_iterate_s, whose
-// operands stay in L2 and whose 1024-thread CTAs meet through atomics: 30.1 -> 17.7 us
-// per pivot at 4096 x 8192, 19.8 -> 9.2 at 701 x 1203, 20.6 -> 9.2 at 200 x 300,
-// 24.3 -> 9.0 on a degenerate 256 x 512 under the safety net.
+// operands stay in L2 and whose 1024-thread CTAs meet through atomics: 30.1 -> 17.0 us
+// per pivot at 4096 x 8192, 19.8 -> 9.0 at 701 x 1203, 20.6 -> 9.0 at 200 x 300,
+// 24.3 -> 9.1 on a degenerate 256 x 512 under the safety net.
 #include "lpgb_internal.cuh"
 #include "struct_common.cuh"
 #include "../../include/lpgb.h"

@@ -1,5 +1,7 @@
 // kernels_struct.cu -- the persistent engine on the slack-structured form of
-// the explicit inverse (engine LP_ENGINE_STRUCTURED).
+// the explicit inverse (engine LP_ENGINE_STRUCTURED).  The pivots run in k_iterate_r
+// (kernels_resident.cu) wherever that applies; k_iterate_s here runs the lexicographic
+// rule, priority lists and the sizes k_iterate_r's layouts do not hold.
 //
 // Let R be the constraint rows whose slack is nonbasic and k = |R|.  With the
 // basis columns ordered as structurals then slacks, B = [[A_RJ, 0], [A_SJ, I]]

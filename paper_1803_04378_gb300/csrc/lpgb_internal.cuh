@@ -193,7 +193,7 @@ struct DevState {
     int32_t* lex_rows;  // m: rows of the ratio-test tie set (lexicographic rule)
     int32_t* crash_list;  // m: the structurals a warm-start crash enters, in order (lp_set_crash)
     uint32_t* gbar;     // k_iterate grid barrier: arrivals, released epoch
-    // slack-structured engine (k_iterate_s): the constraint rows in slot order,
+    // slack-structured engine (k_iterate_r, k_iterate_s): the constraint rows in slot order,
     // the rows whose slack is nonbasic in slots [0, k_live)
     double* A_p;        // n columns of ld doubles: A with its rows in slot order
     float* A_p32;       // its FP32 copy (the PRICE screen)

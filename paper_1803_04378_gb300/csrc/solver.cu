@@ -54,7 +54,7 @@ struct lp_handle {
     bool persist = false;            // pivots run in k_iterate (cooperative, one CTA per SM)
     int persist_blocks = 0;
     cudaEvent_t evc0 = nullptr, evc1 = nullptr;  // kernel_timing around k_iterate launches
-    bool structured = false;         // pivots run in k_iterate_s (LP_ENGINE_STRUCTURED)
+    bool structured = false;         // pivots run in k_iterate_r or k_iterate_s (LP_ENGINE_STRUCTURED)
     int engine_reason = LP_ENGINE_REASON_NONE;  // why the engine that runs is not the one asked for
     // Case 2 (tableau_budget_mb exceeded): B^-1 in pinned host memory, streamed in row blocks
     bool ooc = false;
