@@ -65,6 +65,12 @@ constexpr unsigned kRMore = 1u << 31;  // PRICE record: more than one column lis
 constexpr int kRList = 4;         // columns listed in a PRICE record
 constexpr int kRWarpList = 16;    // columns kept per polling warp
 constexpr int kRCand = 16;        // columns re-priced by every CTA
+// Meetings of one step at most: the PRICE records, the FP64 pricing's where they decide
+// nothing, the ratio test's records, and the two of a scanned tie set (a step that
+// stops or repairs holds one).  A launch holds one more, at its start.  The next
+// launch's numbers begin past all that this one can use: a number already stamped in
+// a mailbox would be taken for an answer without waiting.
+constexpr unsigned kRStepMeetings = 5;
 
 // ---- the meeting of all CTAs ---------------------------------------------------------
 __device__ __forceinline__ void st_relaxed_b128(ulonglong2* p, unsigned long long lo, unsigned long long hi) {
@@ -1244,6 +1250,8 @@ int resident_ctas(int sms, int m, int n) {
     if (g < 56) g = std::min(std::max(g, 16), 32);
     return std::max(1, std::min(std::min(g, std::max(m, n)), std::min(kRMaxCtas, sms)));
 }
+
+unsigned resident_meetings(int iters) { return kRStepMeetings * (unsigned)iters + 1; }
 
 size_t resident_meet_bytes(int ctas) { return sizeof(ulonglong2) * 2 * kRChunks * (size_t)ctas * ctas; }
 

@@ -309,8 +309,8 @@ int resident_ctas(int sms, int m, int n);
 size_t resident_meet_bytes(int ctas);  // the CTAs' records (zero before the first launch)
 // false: not even the vectors fit
 bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t smem_optin, ResidentPlan* out);
-// uses the meeting numbers seq0 + 1 .. seq0 + resident_meetings(iters)
-inline unsigned resident_meetings(int iters) { return 4u * (unsigned)iters + 2u; }
+// uses meeting numbers seq0 + 1 .. seq0 + resident_meetings(iters) at most
+unsigned resident_meetings(int iters);
 cudaError_t launch_iterate_r(const DevState& s, const ResidentPlan& p, int iters, void* meet, unsigned seq0,
                              cudaStream_t st);
 // Bounded-wait self-test: a grid barrier that cannot complete (lp_selftest_barrier_timeout).
