@@ -7,6 +7,7 @@
 // reads the 160-byte control block after each graph launch, and rebuilds B^-1
 // when the device asks for it.
 #include "lpgb_internal.cuh"
+#include "meeting_numbers.hpp"
 #include "../../include/lpgb.h"
 
 #include <algorithm>
@@ -74,7 +75,7 @@ struct lp_handle {
     int r_ctas = 0;                  // k_iterate_r: CTAs per launch
     size_t smem_optin = 0;           // shared memory a block may use
     ulonglong2* r_meet = nullptr;    // k_iterate_r: the CTAs' records
-    unsigned r_seq = 0;              // last meeting number handed out
+    uint32_t r_seq = 0;              // last meeting number handed out
     int32_t* csc_cnt = nullptr;      // price_mode 2: per-column nonzero counts (scratch)
     double chain_s = 0.0, chain_b = 0.0;
     int chain_n = 0;
@@ -510,8 +511,11 @@ bool resident_fits(const lp_handle* h, int k_live, ResidentPlan* rp) {
 // fits one launch).
 cudaError_t launch_resident(lp_handle* h, const ResidentPlan& rp) {
     const int iters = h->opt.graph_iters + 1;
-    const unsigned seq0 = h->r_seq;
-    h->r_seq += resident_meetings(iters);
+    uint32_t seq0 = 0;
+    if (take_meeting_numbers(h->r_seq, resident_meetings(iters), &seq0)) {
+        const cudaError_t e = cudaMemsetAsync(h->r_meet, 0, resident_meet_bytes(h->r_ctas), h->stream);
+        if (e != cudaSuccess) return e;
+    }
     return launch_iterate_r(h->ds, rp, iters, h->r_meet, seq0, h->stream);
 }
 
