@@ -90,7 +90,8 @@ extern "C" {
                                               or its 28 ld bytes of shared memory exceed the
                                               device's per-block limit (m above about 5600 on
                                               152 SMs) */
-#define LP_ENGINE_REASON_OCCUPANCY 5       /* the persistent kernel does not fit one CTA per SM */
+#define LP_ENGINE_REASON_OCCUPANCY 5       /* the persistent kernel does not fit one CTA per SM, or
+                                              a launch of it was refused during a solve */
 #define LP_ENGINE_REASON_OUT_OF_CORE 6     /* tableau_budget_mb: B^-1 streams through the device in row
                                               blocks (Case 2), on the captured-graph engine's kernels */
 

@@ -693,9 +693,9 @@ __global__ void k_barrier_selftest(uint32_t* bar, int32_t* err) {
 size_t price_smem_bytes(int ld) { return (size_t)ld * sizeof(double); }
 size_t update_smem_bytes(int ld) { return 2 * (size_t)ld * sizeof(double); }
 
-void configure_iter_kernels(int ld) {
-    cudaFuncSetAttribute(k_price, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)price_smem_bytes(ld));
-    cudaFuncSetAttribute(k_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)update_smem_bytes(ld));
+void configure_iter_kernels() {
+    raise_smem_limit(reinterpret_cast<const void*>(k_price));
+    raise_smem_limit(reinterpret_cast<const void*>(k_update));
 }
 
 void launch_init_slack(const DevState& s, cudaStream_t st) {
@@ -729,8 +729,8 @@ int occupancy_price(int ld) {
 size_t iterate_smem_bytes(int ld) { return 2 * (size_t)ld * sizeof(double); }
 
 int occupancy_iterate(int ld) {
-    cudaFuncSetAttribute(k_iterate<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)iterate_smem_bytes(ld));
-    cudaFuncSetAttribute(k_iterate<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)iterate_smem_bytes(ld));
+    raise_smem_limit(reinterpret_cast<const void*>(k_iterate<false>));
+    raise_smem_limit(reinterpret_cast<const void*>(k_iterate<true>));
     int nb = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_iterate<false>, kUpdateThreads, iterate_smem_bytes(ld));
     return nb;

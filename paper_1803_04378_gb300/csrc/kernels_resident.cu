@@ -1255,8 +1255,19 @@ unsigned resident_meetings(int iters) { return kRStepMeetings * (unsigned)iters 
 
 size_t resident_meet_bytes(int ctas) { return sizeof(ulonglong2) * 2 * kRChunks * (size_t)ctas * ctas; }
 
-bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t smem_optin, ResidentPlan* out) {
-    constexpr size_t kStatic = 4096;  // static shared memory of the kernel, rounded up
+cudaError_t resident_room(size_t* room) {
+    const ResKernel k[3] = {res_kernel(true, true), res_kernel(true, false), res_kernel(false, false)};
+    *room = SIZE_MAX;
+    for (ResKernel f : k) {
+        size_t r = 0;
+        const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(f), &r);
+        if (e != cudaSuccess) return e;
+        *room = std::min(*room, r);
+    }
+    return cudaSuccess;
+}
+
+bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t room, ResidentPlan* out) {
     // room for every pivot of the launch to add a live slot, and at least one
     const int want = std::min(ld, (k_live + iters + 1 + 63) & ~63);
     for (int v = 0; v < 3; ++v) {
@@ -1264,7 +1275,7 @@ bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t
         const int least = std::min(ld, (k_live + 1 + 63) & ~63);
         for (int kc = want; kc >= least; kc -= 64) {
             const ResLayout l = res_layout(m, n, ctas, kc, a, b);
-            if (l.bytes + kStatic <= smem_optin) {
+            if (l.bytes <= room) {
                 out->ctas = ctas; out->kc = kc; out->a = a; out->b = b; out->smem = l.bytes;
                 return true;
             }
@@ -1276,9 +1287,6 @@ bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t
 cudaError_t launch_iterate_r(const DevState& s, const ResidentPlan& p, int iters, void* meet, unsigned seq0,
                              cudaStream_t st) {
     ResKernel k = res_kernel(p.a, p.b);
-    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)p.smem);
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.ctas);
     cfg.blockDim = dim3(kRThreads);

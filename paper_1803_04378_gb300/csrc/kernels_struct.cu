@@ -1205,7 +1205,7 @@ bool struct_engine_fits(int m, int ld, int ctas) {
 }
 
 int occupancy_iterate_s(int ld) {
-    cudaFuncSetAttribute(k_iterate_s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)iterate_s_smem_bytes(ld));
+    raise_smem_limit(reinterpret_cast<const void*>(k_iterate_s));
     int nb = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_iterate_s, kUpdateThreads, iterate_s_smem_bytes(ld));
     return nb;

@@ -268,6 +268,24 @@ inline cudaError_t launch_k(void (*kernel)(Args...), dim3 grid, dim3 block, size
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Raises a kernel's dynamic shared-memory limit to all that a block may use beside the
+// kernel's static part (*room).  The limit belongs to the function, on its device, and
+// not to a handle: set to one handle's size, a smaller handle made later, or another
+// thread's between this setting and the launch, would have the launch refused.
+// Set to the same value by all, it is safe from any thread; a launch still gets
+// what it asks for and no more.
+inline cudaError_t raise_smem_limit(const void* kernel, size_t* room = nullptr) {
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    int dev = 0, optin = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    const int most = optin - (int)fa.sharedSizeBytes;
+    if (room) *room = (size_t)most;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 struct Geometry {
     int sms;
     int price_blocks, price_threads;
@@ -308,7 +326,8 @@ struct ResidentPlan {
 int resident_ctas(int sms, int m, int n);
 size_t resident_meet_bytes(int ctas);  // the CTAs' records (zero before the first launch)
 // false: not even the vectors fit
-bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t smem_optin, ResidentPlan* out);
+bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t room, ResidentPlan* out);
+cudaError_t resident_room(size_t* room);  // dynamic shared memory of a CTA; opens it to the kernels
 // uses meeting numbers seq0 + 1 .. seq0 + resident_meetings(iters) at most
 unsigned resident_meetings(int iters);
 cudaError_t launch_iterate_r(const DevState& s, const ResidentPlan& p, int iters, void* meet, unsigned seq0,
@@ -317,7 +336,7 @@ cudaError_t launch_iterate_r(const DevState& s, const ResidentPlan& p, int iters
 int barrier_selftest(int blocks, cudaStream_t st);
 size_t price_smem_bytes(int ld);
 size_t update_smem_bytes(int ld);
-void configure_iter_kernels(int ld);
+void configure_iter_kernels();
 
 // ---- sparse copy of A (kernels_sparse.cu) ----------------------------------------
 // cnt: n int32 scratch; ptr: n+1 column starts (ptr[n] = nonzeros).
@@ -339,7 +358,7 @@ void launch_ooc_update(const DevState& s, const Geometry& g, double* win, int i0
 void launch_ooc_chuzr(const DevState& s, cudaStream_t st);
 void launch_ooc_fetch_row(const DevState& s, const double* host_binv, const double* win, int w0, int w1,
                           double* prow, cudaStream_t st);
-int configure_ooc_kernels(int ld);
+int configure_ooc_kernels();
 // sliced FP64 products on the tensor cores (ozaki.cu)
 bool oz_fits(int k);
 size_t oz_scratch_x_elems(int m);

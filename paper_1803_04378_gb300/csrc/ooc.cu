@@ -203,11 +203,8 @@ void launch_ooc_fetch_row(const DevState& s, const double* host_binv, const doub
     k_ooc_fetch_row<<<8, 256, 0, st>>>(s, host_binv, win, w0, w1, prow);
 }
 
-int configure_ooc_kernels(int ld) {
-    return cudaFuncSetAttribute(k_ooc_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)update_smem_bytes(ld)) == cudaSuccess
-               ? 0
-               : -1;
+int configure_ooc_kernels() {
+    return raise_smem_limit(reinterpret_cast<const void*>(k_ooc_update)) == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace lpgb

@@ -73,7 +73,7 @@ struct lp_handle {
     bool s_force = true;             // rebuild the slot map and A_p on the next entry
     int32_t* s_relayout = nullptr;   // device flag: the entry rebuilt the slot map
     int r_ctas = 0;                  // k_iterate_r: CTAs per launch
-    size_t smem_optin = 0;           // shared memory a block may use
+    size_t r_room = 0;               // its dynamic shared memory per CTA
     ulonglong2* r_meet = nullptr;    // k_iterate_r: the CTAs' records
     uint32_t r_seq = 0;              // last meeting number handed out
     int32_t* csc_cnt = nullptr;      // price_mode 2: per-column nonzero counts (scratch)
@@ -188,7 +188,7 @@ int setup_geometry(lp_handle* h) {
     CK(cudaGetDeviceProperties(&prop, h->device));
     Geometry& g = h->geo;
     g.sms = prop.multiProcessorCount;
-    configure_iter_kernels(h->ld);
+    configure_iter_kernels();
     const int occ_p = std::max(1, occupancy_price(h->ld));
     g.price_threads = 1024;
     g.update_threads = 1024;
@@ -503,7 +503,7 @@ int reinvert(lp_handle* h, int check_feasible, bool refine, bool to_struct = fal
 // priority list, which it does not have; vectors that fit in shared memory).
 bool resident_fits(const lp_handle* h, int k_live, ResidentPlan* rp) {
     return !h->p.lex && !h->p.prio &&
-           resident_plan(h->m, h->n, h->ld, h->r_ctas, k_live, h->opt.graph_iters + 1, h->smem_optin, rp);
+           resident_plan(h->m, h->n, h->ld, h->r_ctas, k_live, h->opt.graph_iters + 1, h->r_room, rp);
 }
 
 // Up to graph_iters + 1 of its steps (one more than graph_iters: the first step
@@ -870,7 +870,7 @@ static int create_impl(lp_handle* h, int32_t m, int32_t n, const double* A, cons
             CK(cudaEventCreateWithFlags(&h->ooc_ev_upd[b], cudaEventDisableTiming));
             CK(cudaEventCreateWithFlags(&h->ooc_ev_d2h[b], cudaEventDisableTiming));
         }
-        if (configure_ooc_kernels(ld) != 0) return LP_ERR_CUDA;
+        if (configure_ooc_kernels() != 0) return LP_ERR_CUDA;
     } else {
         TRY(dalloc(h, &binv, (size_t)m * ld));
     }
@@ -999,9 +999,7 @@ static int create_impl(lp_handle* h, int32_t m, int32_t n, const double* A, cons
             TRY(dalloc(h, &h->s_relayout, 1));
             TRY(dalloc(h, &s.price_rec, (size_t)h->geo.sms));
             TRY(dalloc(h, &s.row_rec, (size_t)h->geo.sms));
-            int optin = 0;
-            CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
-            h->smem_optin = (size_t)optin;
+            CK(resident_room(&h->r_room));
             h->r_ctas = resident_ctas(h->geo.sms, m, n);
             TRY(dalloc(h, &h->r_meet, resident_meet_bytes(h->r_ctas) / sizeof(ulonglong2)));
             CK(cudaMemsetAsync(h->r_meet, 0, resident_meet_bytes(h->r_ctas), h->stream));
@@ -1331,6 +1329,7 @@ int lp_solve(lp_handle* h, lp_result* out) {
                 TRY(reinvert_settle(h, rq, &redo));
             }
             h->structured = false;
+            h->engine_reason = LP_ENGINE_REASON_OCCUPANCY;
             TRY(reinvert(h, 0, false));
             continue;
         }
@@ -1362,6 +1361,7 @@ int lp_solve(lp_handle* h, lp_result* out) {
             // the cooperative launch was refused: captured graphs from here on
             (void)cudaGetLastError();
             h->persist = false;
+            h->engine_reason = LP_ENGINE_REASON_OCCUPANCY;
         }
         if (!h->graph) TRY(capture_graph(h));  // on the first use of the captured-graph engine
         CK(cudaGraphLaunch(h->graph, h->stream));
