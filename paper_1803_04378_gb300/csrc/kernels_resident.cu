@@ -16,11 +16,22 @@
 // reinversion reads the whole.  At 4096 x 8192, G = 152 and k = 344 that is
 // 74 KB of A and 74 KB of B^-1 per CTA.
 //
-// Meeting.  The two grid barriers of a pivot carry the CTAs' records: thread c of a
-// CTA puts the record into CTA c's mailbox, each 16-byte chunk stamped with the sequence
-// number of the meeting, and then polls its own mailbox for CTA c's.  Reading every
+// Meeting.  The two grid barriers of a pivot carry the CTAs' records: each goes into
+// every CTA's mailbox, its 16-byte chunks stamped with the sequence number of the
+// meeting, and thread c polls its own CTA's mailbox for CTA c's.  Reading every
 // CTA's record is the barrier, so a meeting costs one store and one load round
 // trip instead of an atomic, a poll and the records' own loads.
+//
+// Order.  The ratio test's meeting publishes what the other CTAs read in the next step:
+// the rows of B^-1, the moved slots of A_p, the tabu list.  The warp that sends its
+// record has fenced first, after a block barrier behind those writes: a fence, then
+// a store of the same thread, is a release for all that the CTA wrote before the
+// barrier, and the polls acquire.  The fence runs beside FTRAN.  (A release in
+// each of the record's stores costs 0.9 to 1.3 us a pivot, a fence in every polling
+// warp 0 to 0.5, this 0 to 0.18.)  So do the repair's meeting and those without a record.
+// The PRICE meeting publishes nothing.  After it the pivot row's owner overwrites the
+// row, which every CTA has read: each record sent is computed from the row's
+// values, so a read that returned the later ones would be the cause of itself.
 //
 // PRICE decides on intervals.  The FP32 screen gives every column an interval
 // that holds its reduced cost.  The record of a CTA is its largest lower end
@@ -58,6 +69,7 @@ namespace {
 constexpr int kRThreads = 512;
 constexpr int kRWarps = kRThreads / 32;
 constexpr int kRPrice = 8;        // warps that screen and poll; the others apply the rank-1 update
+constexpr int kRMail = kRWarps - 1;  // the warp that fences for the CTA and sends what publishes its data
 constexpr int kRMaxCtas = 32 * kRPrice;
 constexpr int kRChunks = 4;       // 16-byte chunks of a record: three payload words and the stamp
 constexpr int kRWords = 3 * kRChunks;
@@ -86,10 +98,10 @@ __device__ __forceinline__ ulonglong2 ld_acquire_b128(const ulonglong2* p) {
 
 // One chunk of the CTA's record under `seq`, into CTA dest's mailbox.  Every CTA has a
 // mailbox of its own, which no other polls, a sender's 16 bytes beside the next
-// sender's: a warp polls 32 senders in four lines, and thread t puts the record into
-// mailbox t.  One record for all, 64 bytes apart and polled by every CTA, held up its writer
-// (17.9 us a pivot against 17.0 at 4096 x 8192 on 152 CTAs, 10.6 against 9.5 at
-// 1024 x 2048); chunks of several CTAs in one line that all poll took 2.3 us a meeting.
+// sender's: a warp polls 32 senders in four lines.  One record for all, 64 bytes apart
+// and polled by every CTA, held up its writer (17.9 us a pivot against 17.0 at
+// 4096 x 8192 on 152 CTAs, 10.6 against 9.5 at 1024 x 2048); chunks of several CTAs in
+// one line that all poll took 2.3 us a meeting.
 __device__ __forceinline__ void meet_put(ulonglong2* buf, unsigned seq, int dest, int chunk, unsigned a, unsigned b,
                                          unsigned c) {
     st_relaxed_b128(buf + (((size_t)(seq & 1) * gridDim.x + dest) * kRChunks + chunk) * gridDim.x + blockIdx.x,
@@ -377,11 +389,12 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
                 for (int t = lane; t < kc; t += 32)
                     Bs[(size_t)l * kc + t] = t < k0 ? __ldcg(s.bp + (size_t)(b + G * l) * ld + t) : 0.0;
     }
-    // a meeting without a record
+    // a meeting without a record (off the chain: each sender fences)
     auto meet = [&] {
         __syncthreads();
         ++seq;
         if (tid < G) {
+            __threadfence();
             meet_put(xbuf, seq, tid, 0, 0, 0, 0);
             unsigned w[3];
             meet_get<0, 1>(xbuf, seq, tid, w, &fail);
@@ -634,7 +647,8 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
             }
             __syncthreads();
             ++seq;
-            if (warp == 0) {
+            if (warp == kRMail) {
+                __threadfence();  // the updated rows
                 const long long klim = dkey(-rep_tol);
                 long long kb = kbig;
                 int pi = INT_MAX, var = 0;
@@ -644,21 +658,17 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
                 }
                 const long long wm = warp_min_key(kb);
                 const int win = warp_argmin_index(pi, kb == wm && wm != kbig);
-                if (lane == 0) __threadfence();  // the updated rows, before the record
-                __syncwarp();
-                if (lane == max(win, 0)) {
-                    rpub[0] = ll_lo(wm); rpub[1] = ll_hi(wm); rpub[2] = (unsigned)(win < 0 ? -1 : pi);
-                    rpub[5] = (unsigned)var;
+                const int pw = __shfl_sync(0xffffffffu, pi, max(win, 0)), vw = __shfl_sync(0xffffffffu, var, max(win, 0));
+                for (int d = lane; d < G; d += 32) {
+                    meet_put(xbuf, seq, d, 0, ll_lo(wm), ll_hi(wm), (unsigned)(win < 0 ? -1 : pw));
+                    meet_put(xbuf, seq, d, 1, 0, 0, (unsigned)vw);
                 }
             }
             if (warp < nwu) {
-                asm volatile("bar.sync 1, %0;\n" ::"r"(32 * nwu) : "memory");
                 unsigned w[kRWords];
                 long long kb = kbig;
                 int pi = INT_MAX, var = 0;
                 if (tid < G) {
-                    meet_put(xbuf, seq, tid, 0, rpub[0], rpub[1], rpub[2]);
-                    meet_put(xbuf, seq, tid, 1, 0, 0, rpub[5]);
                     meet_get<0, 2>(xbuf, seq, tid, w, &fail);
                     kb = words_ll(w[0], w[1]);
                     pi = (int)w[2];
@@ -967,6 +977,7 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
             if (warp < nwu) {
                 unsigned w[kRWords];
                 if (tid < G) {
+                    __threadfence();
                     meet_put(xbuf, seq, tid, 0, ll_lo(cpub.d_all), ll_hi(cpub.d_all), (unsigned)cpub.j_all);
                     meet_put(xbuf, seq, tid, 1, ll_lo(cpub.d_nt), ll_hi(cpub.d_nt), (unsigned)cpub.j_nt);
                     meet_put(xbuf, seq, tid, 2, ll_lo(cpub.d_min), ll_hi(cpub.d_min), (unsigned)cpub.j_min);
@@ -1065,12 +1076,10 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
                     }
                 }
             }
-            // What the other CTAs read after the ratio meeting (the rows of B^-1, the tabu
-            // list) was written before this step's last block barrier.  The fence that
-            // makes it visible runs beside FTRAN, in the warp with the fewest rows,
-            // and the record goes out after the next block barrier: in the record's
-            // own warp it cost 0.6 us of every pivot.
-            if (tid == kRThreads - 1) __threadfence();
+            // What the other CTAs read after the ratio meeting was written before this step's
+            // last block barrier.  The record's warp, which has the fewest rows, fences
+            // here, beside FTRAN: after the next block barrier it cost 0.6 us of every pivot.
+            if (warp == kRMail) __threadfence();
             if (!dq_known && qn < n && warp >= kRWarps - 3 && warp < kRWarps - 1) {
                 // the two row segments of price_block
                 const int nch = kk >> 6, sg = warp - (kRWarps - 3);
@@ -1085,24 +1094,26 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
             }
         }
         __syncthreads();
-        // ---- the CTA's ratio-test record
+        // ---- the CTA's ratio-test record, by the warp that fenced
         ++seq;
-        if (warp == 0) {
+        if (warp == kRMail) {
             ratio_record(P, owned, bland, al, bb, rvar, rpub);
-        } else if (tid == kRThreads - 32 && !dq_known) {
+            __syncwarp();
+            for (int d = lane; d < G; d += 32) {
+                meet_put(xbuf, seq, d, 0, rpub[0], rpub[1], rpub[2]);
+                meet_put(xbuf, seq, d, 1, rpub[3], rpub[4], rpub[5]);
+                if (rpub[5] & kRMore) meet_put(xbuf, seq, d, 2, rpub[6], rpub[7], rpub[8]);
+            }
+        } else if (tid == kRThreads - 64 && !dq_known) {
             S.dq = qn < n ? cq_sh - (dpart[0] + dpart[1]) : -ycur[rs[qn - n]];
         }
         if (warp < nwu) {
-            asm volatile("bar.sync 1, %0;\n" ::"r"(32 * nwu) : "memory");
             unsigned w[kRWords];
             long long tmin = kbig;
             double ra = 0.0;
             int var = 0, row = -1;
             bool more = false;
             if (tid < G) {
-                meet_put(xbuf, seq, tid, 0, rpub[0], rpub[1], rpub[2]);
-                meet_put(xbuf, seq, tid, 1, rpub[3], rpub[4], rpub[5]);
-                if (rpub[5] & kRMore) meet_put(xbuf, seq, tid, 2, rpub[6], rpub[7], rpub[8]);
                 meet_get<0, 2>(xbuf, seq, tid, w, &fail);
                 tmin = words_ll(w[0], w[1]);
                 row = (int)w[2];
@@ -1171,9 +1182,7 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
             __syncthreads();
         }
         if (scan_sh) {
-            // CTAs with other minima lie within the tie tolerance: scan the rows of all
-            // CTAs (alpha and bbar of this step made visible first)
-            if (tid == 0) __threadfence();
+            // CTAs with other minima lie within the tie tolerance: scan the rows of all CTAs
             meet();
             if (fail) break;
             const double thr = tie_limit(thr_sh, P.tol_tie);
