@@ -650,6 +650,12 @@ __device__ bool grid_barrier(uint32_t* bar, unsigned& epoch, volatile int* fail,
     return *fail == 0;
 }
 
+// Any CTA that gave up a wait reports it: the others, the lead CTA among them, may have
+// ended theirs in time, and what this one leaves undone is then theirs to read.
+__device__ __forceinline__ void report_timeout(int fail, int32_t* err) {
+    if (threadIdx.x == 0 && fail) atomicExch(err, kErrTimeout);
+}
+
 // Step 7/8 bookkeeping of the pivot (q, r): identical scalar updates in every
 // CTA; the lead CTA also writes the basis exchange, tabu list, trace and
 // counters (the same rules as k_pivot).

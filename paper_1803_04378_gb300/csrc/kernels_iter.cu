@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(kUpdateThreads, 1) k_iterate(DevState s, int i
     }
     // every CTA has its copy of the control block before block 0 changes it
     if (!grid_barrier(s.gbar, epoch, &fail)) {
-        if (lead && threadIdx.x == 0) C->err = kErrTimeout;
+        report_timeout(fail, &C->err);
         return;
     }
     for (int step = 0; step < iters; ++step) {
@@ -671,10 +671,8 @@ __global__ void __launch_bounds__(kUpdateThreads, 1) k_iterate(DevState s, int i
         __syncthreads();
         if (S.status != kRunning) break;
     }
-    if (lead && threadIdx.x == 0) {
-        iterate_flush(s, S);
-        if (fail) C->err = kErrTimeout;
-    }
+    if (lead && threadIdx.x == 0) iterate_flush(s, S);
+    report_timeout(fail, &C->err);
 }
 
 // Self-test of the bounded wait: the barrier expects one CTA more than the
@@ -754,15 +752,12 @@ cudaError_t launch_iterate(const DevState& s, int blocks, int iters, cudaStream_
 }
 
 int barrier_selftest(int blocks, cudaStream_t st) {
+    // the barrier's two words, the two tests' error words, the meeting's mailboxes
     uint32_t* bar = nullptr;
-    int32_t* err = nullptr;
-    if (cudaMallocAsync(&bar, 2 * sizeof(uint32_t), st) != cudaSuccess) return LP_ERR_CUDA;
-    if (cudaMallocAsync(&err, sizeof(int32_t), st) != cudaSuccess) {
-        cudaFreeAsync(bar, st);
-        return LP_ERR_CUDA;
-    }
-    cudaMemsetAsync(bar, 0, 2 * sizeof(uint32_t), st);
-    cudaMemsetAsync(err, 0, sizeof(int32_t), st);
+    const size_t words = 4 * sizeof(uint32_t), bytes = words + resident_meet_bytes(blocks);
+    if (cudaMallocAsync(&bar, bytes, st) != cudaSuccess) return LP_ERR_CUDA;
+    int32_t* err = reinterpret_cast<int32_t*>(bar + 2);
+    cudaMemsetAsync(bar, 0, bytes, st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(32);
@@ -773,14 +768,14 @@ int barrier_selftest(int blocks, cudaStream_t st) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, k_barrier_selftest, bar, err);
-    int32_t h = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = launch_meeting_selftest(blocks, bar + 4, err + 1, st);
+    int32_t h[2] = {};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, err, sizeof(h), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFreeAsync(bar, st);
-    cudaFreeAsync(err, st);
     cudaStreamSynchronize(st);
     if (e != cudaSuccess) return LP_ERR_CUDA;
-    return h == kErrTimeout ? LP_ERR_TIMEOUT : LP_OK;
+    return h[0] == kErrTimeout && h[1] == kErrTimeout ? LP_ERR_TIMEOUT : LP_OK;
 }
 
 int occupancy_update(int ld) {

@@ -1234,9 +1234,25 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
                 C->repair = rep_code;
                 C->repair_end = rep_end;
             }
-            if (fail) C->err = kErrTimeout;
         }
     }
+    report_timeout(fail, &C->err);
+}
+
+// Self-test of the bounded meeting: CTA 0's record for the last CTA is never sent, so that
+// CTA alone must give up after the spin limit and report it.
+__global__ void k_meeting_selftest(ulonglong2* xbuf, int32_t* err) {
+    __shared__ volatile int fail;
+    const int tid = threadIdx.x, G = gridDim.x;
+    if (tid == 0) fail = 0;
+    __syncthreads();
+    if (tid < G) {
+        if (blockIdx.x != 0 || tid != G - 1) meet_put(xbuf, 1, tid, 0, 0, 0, 0);
+        unsigned w[3];
+        meet_get<0, 1>(xbuf, 1, tid, w, &fail);
+    }
+    __syncthreads();
+    report_timeout(fail, err);
 }
 
 using ResKernel = void (*)(DevState, int, int, ulonglong2*, unsigned);
@@ -1245,6 +1261,19 @@ ResKernel res_kernel(bool a, bool b) {
 }
 
 }  // namespace
+
+cudaError_t launch_meeting_selftest(int blocks, void* meet, int32_t* err, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3((blocks + 31) / 32 * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_meeting_selftest, static_cast<ulonglong2*>(meet), err);
+}
 
 // CTAs of a launch.  A CTA's share of the screen, the update and FTRAN falls with
 // the number of CTAs, and the two meetings of a pivot grow with it (one warp polls

@@ -698,7 +698,7 @@ __global__ void __launch_bounds__(kUpdateThreads, 1) k_iterate_s(DevState s, int
         list_ok = 0;
     }
     if (!grid_barrier(s.gbar, epoch, &fail)) {
-        if (lead && threadIdx.x == 0) C->err = kErrTimeout;
+        report_timeout(fail, &C->err);
         return;
     }
     const bool screen_ok = screen_sh != 0;
@@ -1019,10 +1019,8 @@ __global__ void __launch_bounds__(kUpdateThreads, 1) k_iterate_s(DevState s, int
             __syncthreads();
         }
     }
-    if (lead && threadIdx.x == 0) {
-        iterate_flush(s, S);
-        if (fail) C->err = kErrTimeout;
-    }
+    if (lead && threadIdx.x == 0) iterate_flush(s, S);
+    report_timeout(fail, &C->err);
 }
 
 // ---- entering the structured form from the dense state ------------------------------

@@ -332,7 +332,9 @@ cudaError_t resident_room(size_t* room);  // dynamic shared memory of a CTA; ope
 unsigned resident_meetings(int iters);
 cudaError_t launch_iterate_r(const DevState& s, const ResidentPlan& p, int iters, void* meet, unsigned seq0,
                              cudaStream_t st);
-// Bounded-wait self-test: a grid barrier that cannot complete (lp_selftest_barrier_timeout).
+cudaError_t launch_meeting_selftest(int blocks, void* meet, int32_t* err, cudaStream_t st);  // meet: zero
+// Bounded-wait self-tests: a grid barrier that cannot complete, a meeting that one CTA
+// waits for in vain (lp_selftest_barrier_timeout).
 int barrier_selftest(int blocks, cudaStream_t st);
 size_t price_smem_bytes(int ld);
 size_t update_smem_bytes(int ld);

@@ -373,8 +373,8 @@ class LP:
 
 
 def selftest_barrier_timeout(blocks: int = 4, stream=None) -> int:
-    """lp_selftest_barrier_timeout: return code of a grid barrier that cannot
-    complete (LP_ERR_TIMEOUT when its bounded wait works)."""
+    """lp_selftest_barrier_timeout: return code of a grid barrier and a meeting
+    that cannot complete (LP_ERR_TIMEOUT when both waits are bounded and reported)."""
     st = None if stream is None else ctypes.c_void_p(stream)
     return _lib.lp_selftest_barrier_timeout(int(blocks), st)
 
