@@ -136,7 +136,13 @@ __device__ __forceinline__ void block_best(long long key, int j, Red& R, long lo
 // SM at m = 225, k = 25; 65% of the time on 4096 LPs) and, with few LPs, the latency of
 // a pivot (7.8 us at m <= 128).  Against the dense m x m inverse: 4096 LPs
 // of m 16..256 30.6 -> 3.3 ms, 48 LPs of m 16..128 1.04 -> 0.39 ms, the same pivots.
-template <int T>
+// LPs whose rows all become live (k = m), the dense inverse's best case: 1024 of
+// m 128..256 114 -> 78 ms, 48 of m 100..128 4.0 -> 3.7, 48 of m 60..64 1.10 -> 0.98.
+//
+// kPair (2 m <= T): two lanes per row, lane 2 i for the even live columns of row i and lane
+// 2 i + 1 for the odd ones, which are FTRAN's two sums anyway; a thread per row
+// leaves half of the warps idle (the 48 LPs of m 60..64: 1.14 ms).
+template <int T, bool kPair>
 __device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, double* slot, int mmax, int nmax, int ks) {
     const BatchParams& P = s.p;
     const BatchLP L = s.lps[lp];
@@ -147,7 +153,7 @@ __device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, doub
     const double* c = s.c + L.c_off;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int W = T / 32;
-    constexpr int VR = (kBatchMaxM + T - 1) / T;  // rows and columns per thread
+    constexpr int VR = kPair ? 1 : (kBatchMaxM + T - 1) / T;  // rows and columns per thread
     constexpr int VC = (kBatchMaxN + T - 1) / T;
 
     // shared-memory carve-up (sizes by the bucket's largest LP)
@@ -175,6 +181,8 @@ __device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, doub
 
     __shared__ LPScal S;
     __shared__ Red R;
+    const int half = kPair ? tid & 1 : 0;
+    auto row_of = [&](int v) { return kPair ? tid >> 1 : tid + T * v; };
     const long long ktol = dkey(P.tol_d), kpiv = dkey(P.tol_piv), kbig = dkey(DBL_MAX);
 
     // Step 1: slack basis
@@ -391,22 +399,32 @@ __device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, doub
         long long kth[VR], kmin = kbig;
 #pragma unroll
         for (int v = 0; v < VR; ++v) {
-            const int i = tid + T * v;
+            const int i = row_of(v);
             double a0 = 0.0, a1 = 0.0;
             kth[v] = kbig;
             al[v] = th[v] = 0.0;
             if (i < m) {
-                int t = 0;
-#pragma unroll 2
-                for (; t + 1 < k; t += 2) {
-                    a0 = fma(col(t)[i], aq[t], a0);
-                    a1 = fma(col(t + 1)[i], aq[t + 1], a1);
+                const double unit = q < n && basis[i] >= n ? au[i] : 0.0;
+                if (kPair) {
+#pragma unroll 4
+                    for (int t = half; t < k; t += 2) a0 = fma(col(t)[i], aq[t], a0);
+                    if (half) a0 += unit;
+                } else {
+                    int t = 0;
+#pragma unroll 4
+                    for (; t + 1 < k; t += 2) {
+                        a0 = fma(col(t)[i], aq[t], a0);
+                        a1 = fma(col(t + 1)[i], aq[t + 1], a1);
+                    }
+                    if (t < k) a0 = fma(col(t)[i], aq[t], a0);
+                    a1 += unit;
                 }
-                if (t < k) a0 = fma(col(t)[i], aq[t], a0);
-                if (q < n && basis[i] >= n) a1 += au[i];
+            }
+            if (kPair) a1 = __shfl_xor_sync(0xffffffffu, a0, 1);
+            if (i < m) {
                 al[v] = a0 + a1;
-                // ratios one row per lane: a warp-wide division covers 32 rows
-                if (dkey(al[v]) > kpiv) {
+                // ratios one row per lane: a warp-wide division covers its rows
+                if (!half && dkey(al[v]) > kpiv) {
                     th[v] = bbar[i] / al[v];
                     kth[v] = dkey(th[v]);
                 }
@@ -437,11 +455,11 @@ __device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, doub
 #pragma unroll
             for (int v = 0; v < VR; ++v)
                 if (kth[v] <= kthr && kth[v] != kbig) {
-                    const int x = basis[tid + T * v];
+                    const int x = basis[row_of(v)];
                     const long long kv = dkey(al[v]);
                     ++cnt;
                     if (row < 0 || (bland ? x < var : (kv > ka || (kv == ka && x < var)))) {
-                        ka = kv; var = x; row = tid + T * v; bt = th[v]; ba = al[v];
+                        ka = kv; var = x; row = row_of(v); bt = th[v]; ba = al[v];
                     }
                 }
             const unsigned bal = __ballot_sync(0xffffffffu, row >= 0);
@@ -518,15 +536,28 @@ __device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, doub
         // ---- Step 8: own rows of bbar and of the live columns
 #pragma unroll
         for (int v = 0; v < VR; ++v) {
-            const int i = tid + T * v;
+            const int i = row_of(v);
             if (i >= m) continue;
             const double na = -al[v];
-            bbar[i] = i == r ? theta : __dsub_rn(bbar[i], __dmul_rn(al[v], theta));
-#pragma unroll 4
-            for (int t = 0; t < kn; ++t) {
-                const double old = t == J ? 0.0 : col(t == te && src >= 0 ? src : t)[i];
+            if (!half) bbar[i] = i == r ? theta : __dsub_rn(bbar[i], __dmul_rn(al[v], theta));
+            const double moved = src >= 0 ? col(src)[i] : 0.0;  // goes to slot te
+            auto next = [&](int t, double o) {
+                const double old = t == J ? 0.0 : (t == te && src >= 0 ? moved : o);
                 col(t)[i] = i == r ? rho[t] : fma(na, rho[t], old);
+            };
+            // Four loads ahead of their stores: one by one each waits for the store before it,
+            // which may alias it for all the compiler knows (1024 LPs of m 128..256, k = m:
+            // 87 -> 78 ms; eight loads spill, 81).
+            constexpr int st = kPair ? 2 : 1;
+            int t = half;
+            for (; t + 3 * st < kn; t += 4 * st) {
+                double o[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) o[u] = col(t + u * st)[i];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) next(t + u * st, o[u]);
             }
+            for (; t < kn; t += st) next(t, col(t)[i]);
         }
         __syncthreads();
         // ---- periodic reinversion (structure-aware, as in the single-LP solver)
@@ -632,7 +663,7 @@ __device__ void solve_one(const BatchState& s, int lp, unsigned char* smem, doub
     __syncthreads();
 }
 
-template <int T>
+template <int T, bool kPair>
 __global__ void __launch_bounds__(T, 1024 / T) k_batch(BatchState s, int bucket, int begin, int count, int mmax, int nmax,
                                                        int ks) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -644,7 +675,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_batch(BatchState s, int bucket,
         const int k = next;
         __syncthreads();
         if (k >= count) break;
-        solve_one<T>(s, s.order[begin + k], smem, slot, mmax, nmax, ks);
+        solve_one<T, kPair>(s, s.order[begin + k], smem, slot, mmax, nmax, ks);
     }
 }
 
@@ -661,11 +692,13 @@ size_t batch_smem_bytes(int mmax, int nmax, int ks) {
 
 using BatchKernel = void (*)(BatchState, int, int, int, int, int, int);
 
-BatchKernel batch_kernel(int threads) {
+// m: the largest of the launch
+BatchKernel batch_kernel(int threads, int m) {
+    const bool pair = 2 * m <= threads;
     switch (threads) {
-        case 128: return k_batch<128>;
-        case 256: return k_batch<256>;
-        default: return k_batch<512>;
+        case 128: return pair ? k_batch<128, true> : k_batch<128, false>;
+        case 256: return pair ? k_batch<256, true> : k_batch<256, false>;
+        default: return pair ? k_batch<512, true> : k_batch<512, false>;
     }
 }
 
@@ -688,7 +721,10 @@ struct lp_batch {
     int bucket_begin[kBuckets + 1] = {};
     int bucket_m[kBuckets] = {}, bucket_n[kBuckets] = {};  // the largest m and n in each bucket
     // 4096 LPs of m 16..256: 3.31 ms (3.35 with 256 threads throughout, 4.05 with 128, 5.2
-    // with 512; shared-memory columns 3.43); m 16..64 alone 0.44 ms (0.65 with 256)
+    // with 512; shared-memory columns 3.43); m 16..64 alone 0.44 ms (0.65 with 256).
+    // These are for k far below m.  Rows that all become live want more threads (1024 LPs
+    // of m 65..128 11.6 ms with 128, 7.7 with 256, 8.8 with 512; 512 of m 193..256 119, 74,
+    // 51): lp_batch_tune finds them on the batch itself.
     int cfg_threads[kBuckets] = {128, 128, 256, 256};
     int cfg_smem[kBuckets] = {0, 0, 0, 0};
     int64_t sum_m = 0, sum_n = 0;
@@ -748,7 +784,7 @@ int grid_for(const lp_batch* h, int bucket, int* grid, size_t* smem) {
     const int T = h->cfg_threads[bucket];
     const bool sm = h->cfg_smem[bucket] != 0;
     *smem = batch_smem_bytes(h->bucket_m[bucket], h->bucket_n[bucket], sm ? kSmemCols : 0);
-    BatchKernel k = batch_kernel(T);
+    BatchKernel k = batch_kernel(T, h->bucket_m[bucket]);
     // (one limit for every bucket: buckets with the same thread count share a kernel)
     BCK(cudaFuncSetAttribute(reinterpret_cast<const void*>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)batch_smem_bytes(kBatchMaxM, kBatchMaxN, kSmemCols)));
@@ -791,7 +827,7 @@ int launch_buckets(lp_batch* h, int b0, int b1, const BucketLaunch* plan, bool c
             st = h->bstream[bk];
             BCK(cudaStreamWaitEvent(st, h->fork, 0));
         }
-        BatchKernel k = batch_kernel(h->cfg_threads[bk]);
+        BatchKernel k = batch_kernel(h->cfg_threads[bk], h->bucket_m[bk]);
         k<<<plan[bk].grid, h->cfg_threads[bk], plan[bk].smem, st>>>(h->st, bk, begin, cnt, h->bucket_m[bk], h->bucket_n[bk],
                                                                     h->cfg_smem[bk] ? kSmemCols : 0);
         BCK(cudaGetLastError());
