@@ -504,7 +504,7 @@ __global__ void k_refine_extract(DevState s, int k, int from_struct, int k_live,
 // kMode 2: Y1[i][c] = Y0[i][c] + sum_l Y0[i][l] R[l][c], into rv_W; the first column of
 //          tiles sums the partials (in tile order) into ||R||_inf, as k_refine_finish_residual.
 // Each output is one chain in increasing l, so the result does not depend on the launch
-// shape.  R's sum runs beside a bias, which holds every addend to a multiple of
+// shape.  kComp: R's sum runs beside a bias, which holds every addend to a multiple of
 // 2^-32 as long as the sum stays below 2^19; what that cuts off each product (exact: a
 // fused multiply-add of it) goes into a second sum.  So R has no rounding error to
 // speak of, and Y1 little more than that of its last addition: with these sums at every k, x
@@ -518,10 +518,13 @@ __global__ void k_refine_extract(DevState s, int k, int from_struct, int k_live,
 // k = 32, 64, 96, 128: 15, 22, 30-56, 35-72 here (tiles then share SMs),
 // 31, 32, 36, 36 sliced.
 // kRefineDense: where 3 k^2 > m^2, these products up to this k (refine_fits).
+// Beyond both, where the slices are switched off or past their largest k, the FP64 pipe
+// bounds the products (2 k^3 operations with plain sums, 5 k^3 with kComp) and R's sums
+// are plain: one refinement at k = 1500 takes 12.0 ms, 32 with kComp, an elimination 12.8.
 constexpr int kRefineFp64 = 64, kRefineDense = 256;
 constexpr int kRT = 8, kRC = 64;
 constexpr double kRBias = 1.5 * (1 << 20);
-template <int kMode>
+template <int kMode, bool kComp>
 __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int k_live, int par) {
     pdl_enter();
     if (s.ctrl->err != kErrNone) return;
@@ -575,7 +578,7 @@ __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int
         }
     };
     fetch(0);
-    double acc = kMode == 2 ? 0.0 : kRBias, lo = 0.0;
+    double acc = kComp ? kRBias : 0.0, lo = 0.0;
     for (int l0 = 0; l0 < k; l0 += kRC) {
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
@@ -591,7 +594,7 @@ __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int
             for (int l = l1; l < l1 + 16; ++l) {
                 const double x = xs[ty][l], z = zs[l][tx];
                 const double t = fma(x, z, acc);
-                if (kMode != 2) lo += fma(x, z, acc - t);
+                if (kComp) lo += fma(x, z, acc - t);
                 acc = t;
             }
         __syncthreads();
@@ -608,7 +611,7 @@ __global__ void __launch_bounds__(kRT* kRT) k_refine_fp64(DevState s, int k, int
     }
     double v = 0.0;
     if (in) {
-        v = ((i == c ? 1.0 : 0.0) - (acc - kRBias)) - lo;
+        v = kComp ? ((i == c ? 1.0 : 0.0) - (acc - kRBias)) - lo : (i == c ? 1.0 : 0.0) - acc;
         R[(size_t)i * k + c] = v;
     }
     zs[ty][tx] = fabs(v);
@@ -970,8 +973,8 @@ int launch_refine(const DevState& s, int k, int from_struct, int k_live, int par
     const dim3 tiles(nt, nt), tile(kRT * kRT);
     const bool fp64 = k <= kRefineFp64 || 3 * kk > (size_t)s.p.m * s.p.m;
     if (from_struct && fp64) {
-        launch_k(k_refine_fp64<1>, tiles, tile, 0, st, true, s, k, k_live, par);
-        launch_k(k_refine_fp64<2>, tiles, tile, 0, st, true, s, k, k_live, par);
+        launch_k(k_refine_fp64<1, true>, tiles, tile, 0, st, true, s, k, k_live, par);
+        launch_k(k_refine_fp64<2, false>, tiles, tile, 0, st, true, s, k, k_live, par);
         return 2;
     }
     int blocks = (int)((kk + 255) / 256);
@@ -988,8 +991,8 @@ int launch_refine(const DevState& s, int k, int from_struct, int k_live, int par
         }
     }
     (void)cudaGetLastError();
-    launch_k(k_refine_fp64<0>, tiles, tile, 0, st, true, s, k, k_live, par);
-    launch_k(k_refine_fp64<2>, tiles, tile, 0, st, true, s, k, k_live, par);
+    launch_k(fp64 ? k_refine_fp64<0, true> : k_refine_fp64<0, false>, tiles, tile, 0, st, true, s, k, k_live, par);
+    launch_k(k_refine_fp64<2, false>, tiles, tile, 0, st, true, s, k, k_live, par);
     return 3;
 }
 
