@@ -201,11 +201,12 @@ typedef struct lp_result {
  * lp_selftest_barrier_timeout -- checks the bounded waits of the persistent
  * engines (no counterpart in the paper): a cooperative grid of `blocks` CTAs
  * (1..64) waits at a barrier that expects one CTA more than it has, and one CTA
- * of another waits for a record that is never sent.  They give up after
- * their spin limits (about 2 s), so the call returns LP_ERR_TIMEOUT and the
- * context stays usable; LP_OK would mean that a wait ended without its
- * barrier completing or that a timeout went unreported, LP_ERR_CUDA a refused
- * launch.
+ * of another waits for a record that is never sent; then the lanes of a warp wait
+ * with different limits.  They give up after their spin limits (about 2 s),
+ * so the call returns LP_ERR_TIMEOUT and the context stays usable; LP_OK would
+ * mean that a wait ended without its barrier completing, that a timeout went
+ * unreported or that the warp's lanes got different answers, LP_ERR_CUDA a
+ * refused launch.
  * Synchronizes `cuda_stream` (NULL = default stream).
  */
 int lp_selftest_barrier_timeout(int32_t blocks, void* cuda_stream);

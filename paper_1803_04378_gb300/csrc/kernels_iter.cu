@@ -752,9 +752,9 @@ cudaError_t launch_iterate(const DevState& s, int blocks, int iters, cudaStream_
 }
 
 int barrier_selftest(int blocks, cudaStream_t st) {
-    // the barrier's two words, the two tests' error words, the meeting's mailboxes
+    // the barrier's two words, the three tests' error words, the meeting's mailboxes
     uint32_t* bar = nullptr;
-    const size_t words = 4 * sizeof(uint32_t), bytes = words + resident_meet_bytes(blocks);
+    const size_t words = 8 * sizeof(uint32_t), bytes = words + resident_meet_bytes(blocks);
     if (cudaMallocAsync(&bar, bytes, st) != cudaSuccess) return LP_ERR_CUDA;
     int32_t* err = reinterpret_cast<int32_t*>(bar + 2);
     cudaMemsetAsync(bar, 0, bytes, st);
@@ -768,14 +768,15 @@ int barrier_selftest(int blocks, cudaStream_t st) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, k_barrier_selftest, bar, err);
-    if (e == cudaSuccess) e = launch_meeting_selftest(blocks, bar + 4, err + 1, st);
-    int32_t h[2] = {};
+    if (e == cudaSuccess) e = launch_meeting_selftest(blocks, bar + 8, err + 1, st);
+    if (e == cudaSuccess) e = launch_wait_selftest(err + 2, st);
+    int32_t h[3] = {};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, err, sizeof(h), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFreeAsync(bar, st);
     cudaStreamSynchronize(st);
     if (e != cudaSuccess) return LP_ERR_CUDA;
-    return h[0] == kErrTimeout && h[1] == kErrTimeout ? LP_ERR_TIMEOUT : LP_OK;
+    return h[0] == kErrTimeout && h[1] == kErrTimeout && h[2] == kErrTimeout ? LP_ERR_TIMEOUT : LP_OK;
 }
 
 int occupancy_update(int ld) {

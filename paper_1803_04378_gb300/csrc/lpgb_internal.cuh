@@ -333,8 +333,9 @@ unsigned resident_meetings(int iters);
 cudaError_t launch_iterate_r(const DevState& s, const ResidentPlan& p, int iters, void* meet, unsigned seq0,
                              cudaStream_t st);
 cudaError_t launch_meeting_selftest(int blocks, void* meet, int32_t* err, cudaStream_t st);  // meet: zero
+cudaError_t launch_wait_selftest(int32_t* err, cudaStream_t st);  // *err: kErrTimeout where it holds
 // Bounded-wait self-tests: a grid barrier that cannot complete, a meeting that one CTA
-// waits for in vain (lp_selftest_barrier_timeout).
+// waits for in vain, a warp whose lanes give up at different times (lp_selftest_barrier_timeout).
 int barrier_selftest(int blocks, cudaStream_t st);
 size_t price_smem_bytes(int ld);
 size_t update_smem_bytes(int ld);

@@ -85,6 +85,37 @@ bool tc_make_map_16bit_k(CUtensorMap* map, const void* base, int rows, int cols,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Self-test of the warp's bounded wait: half of warp 0's lanes may try once only, the phase
+// completes 20 ms later (bounded), and all lanes must get one answer; once more with
+// the phase complete.
+__global__ void k_wait_selftest(int32_t* err) {
+    __shared__ uint64_t bar;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        tc::mbar_init(&bar, 1);
+        tc::fence_barrier_init();
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned got = __ballot_sync(0xffffffffu, tc::mbar_wait_warp(&bar, 0, lane < 16 ? 1 : tc::kSpinLimit));
+        const unsigned done = __ballot_sync(0xffffffffu, tc::mbar_wait_warp(&bar, 0));
+        if (lane == 0 && (got == 0 || got == 0xffffffffu) && done == 0xffffffffu) *err = kErrTimeout;
+    } else if (lane == 0) {
+        unsigned long long t0, t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+        for (int i = 0; i < (1 << 22); ++i) {
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (t - t0 > 20000000ull) break;
+        }
+        tc::mbar_arrive(&bar);
+    }
+}
+
+cudaError_t launch_wait_selftest(int32_t* err, cudaStream_t st) {
+    k_wait_selftest<<<1, 64, 0, st>>>(err);
+    return cudaGetLastError();
+}
+
 // D (M x N, FP32, row stride ldd) = A (M x K, row stride lda) * B (N x K, row
 // stride ldb)^T; 16-bit operands, lda and ldb multiples of 8, bases 16-byte
 // aligned.  Returns cudaErrorInvalidValue for shapes or pointers the tensor

@@ -111,9 +111,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const uint32_t tx = (uint32_t)(KB * (a_rows * kTK * 2 + L::kB));
         int s = 0, issued = 0;
         uint32_t ph = 1;
+        bool ok = true;
         for (int t = 0; t < ns; ++t) {
-            if (t >= nst && !tc::mbar_wait(&empty[s], ph)) {
-                fail = 1;
+            if (t >= nst && !tc::mbar_wait_warp(&empty[s], ph)) {
+                ok = false;
                 break;
             }
             uint8_t* sa = smem + s * stage;
@@ -134,15 +135,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             ++issued;
             if (++s == nst) { s = 0; ph ^= 1; }
         }
-        if (fail)  // the loads in flight land before the CTA leaves
-            for (int t = issued > nst ? issued - nst : 0; t < issued; ++t) (void)tc::mbar_wait(&full[t % nst], (t / nst) & 1);
+        if (!ok) {
+            // the loads in flight land before the CTA leaves
+            fail = 1;
+            for (int t = issued > nst ? issued - nst : 0; t < issued; ++t)
+                (void)tc::mbar_wait_warp(&full[t % nst], (t / nst) & 1);
+        }
     } else if (warp == 1) {
         const bool one = tc::elect_one();
         constexpr uint32_t idesc = tc::idesc_f16(kTM, BN, kBF16);
         int s = 0;
         uint32_t ph = 0;
         for (int t = 0; t < ns; ++t) {
-            if (!tc::mbar_wait(&full[s], ph)) {
+            if (!tc::mbar_wait_warp(&full[s], ph)) {
                 fail = 1;
                 break;
             }
@@ -161,7 +166,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
         if (one) tc::mma_commit(tfull);
     } else {
-        if (!tc::mbar_wait(tfull, 0)) {
+        if (!tc::mbar_wait_warp(tfull, 0)) {
             fail = 1;
         } else {
             tc::tc_fence_after();
@@ -224,6 +229,7 @@ __global__ void __launch_bounds__(gemm_p_threads<kEpiWarps>(), kCtas)
     uint64_t* mdone = tempty + 2;       // 1: every MMA of the CTA has completed
     uint32_t* tholder = reinterpret_cast<uint32_t*>(mdone + 1);
     __shared__ volatile int fail;  // read by the other roles' loops: an early way out after a timeout
+    auto gave_up = [&] { return __any_sync(0xffffffffu, fail != 0); };  // (one answer per warp)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nk = (K + kTK - 1) / kTK;
     const int ntn = (N + BN - 1) / BN, ntiles = ntn * ((M + kTM - 1) / kTM);
@@ -254,10 +260,10 @@ __global__ void __launch_bounds__(gemm_p_threads<kEpiWarps>(), kCtas)
         }
         int g = 0, s = 0;  // loads so far, across the CTA's tiles; stage-ring position
         uint32_t ph = 1;
-        for (int t = blockIdx.x; t < ntiles && !fail; t += gridDim.x) {
+        for (int t = blockIdx.x; t < ntiles && !gave_up(); t += gridDim.x) {
             const int m0 = (t / ntn) * kTM, n0 = (t % ntn) * BN;
             for (int kb = 0; kb < nk; ++kb, ++g) {
-                if (g >= kStages && !tc::mbar_wait(&empty[s], ph)) {
+                if (g >= kStages && !tc::mbar_wait_warp(&empty[s], ph)) {
                     fail = 1;
                     break;
                 }
@@ -271,19 +277,19 @@ __global__ void __launch_bounds__(gemm_p_threads<kEpiWarps>(), kCtas)
                 if (++s == kStages) { s = 0; ph ^= 1; }
             }
         }
-        if (fail) {
+        if (gave_up()) {
             // the loads in flight land before the CTA leaves
             for (int h = g - kStages; h < g; ++h)
-                if (h >= 0) (void)tc::mbar_wait(&full[h % kStages], (h / kStages) & 1);
+                if (h >= 0) (void)tc::mbar_wait_warp(&full[h % kStages], (h / kStages) & 1);
         }
     } else if (warp == 1) {
         const bool one = tc::elect_one();
         constexpr uint32_t idesc = tc::idesc_f16(kTM, BN, kBF16);
         int s = 0, i = 0;
         uint32_t ph = 0;
-        for (int t = blockIdx.x; t < ntiles && !fail; t += gridDim.x, ++i) {
+        for (int t = blockIdx.x; t < ntiles && !gave_up(); t += gridDim.x, ++i) {
             const int a = i & 1;
-            if (i >= 2 && !tc::mbar_wait(&tempty[a], ((i >> 1) - 1) & 1)) {
+            if (i >= 2 && !tc::mbar_wait_warp(&tempty[a], ((i >> 1) - 1) & 1)) {
                 fail = 1;
                 break;
             }
@@ -291,7 +297,7 @@ __global__ void __launch_bounds__(gemm_p_threads<kEpiWarps>(), kCtas)
             const uint32_t acc = tmem + (uint32_t)(a * BN);
             bool ok = true;
             for (int kb = 0; kb < nk; ++kb) {
-                if (!tc::mbar_wait(&full[s], ph)) {
+                if (!tc::mbar_wait_warp(&full[s], ph)) {
                     fail = 1;
                     ok = false;
                     break;
@@ -315,15 +321,15 @@ __global__ void __launch_bounds__(gemm_p_threads<kEpiWarps>(), kCtas)
         // every MMA issued by this CTA has completed before the TMEM is freed
         if (one) tc::mma_commit(mdone);
         __syncwarp();
-        if (!tc::mbar_wait(mdone, 0)) fail = 1;
+        if (!tc::mbar_wait_warp(mdone, 0)) fail = 1;
     } else {
         const int lg = warp & 3;  // TMEM lane group of this warp
         const int trow = lg * 32 + lane;
         const int cfirst = 32 * ((warp - 2) >> 2);  // the quarter's warps take chunks cfirst, + 32 kEpiPerQuarter, ...
         int i = 0;
-        for (int t = blockIdx.x; t < ntiles && !fail; t += gridDim.x, ++i) {
+        for (int t = blockIdx.x; t < ntiles && !gave_up(); t += gridDim.x, ++i) {
             const int a = i & 1;
-            if (!tc::mbar_wait(&tfull[a], (i >> 1) & 1)) {
+            if (!tc::mbar_wait_warp(&tfull[a], (i >> 1) & 1)) {
                 fail = 1;
                 break;
             }
