@@ -64,6 +64,11 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// v != 0 (a NaN is), by its bits: an FP64 compare costs the pipe as much as an FMA.
+__device__ __forceinline__ bool nonzero(double v) {
+    return ((unsigned long long)__double_as_longlong(v) << 1) != 0;
+}
+
 // Block-wide best (d, j); valid in thread 0.
 __device__ void block_best(double& d, int& j) {
     __shared__ double sd[32];
@@ -87,9 +92,67 @@ __device__ void block_best(double& d, int& j) {
 // only the rows with a nonzero y_i are read when they are few.  The dense pass is
 // bound by the FP64 pipe (an FMA per 8 bytes): 82 us a call at 4096 x 8192.  With one
 // row in twelve the list takes a twelfth of the FMAs and, in 128-byte pieces, 202 of
-// A's 268 MB: 52 us, bound by DRAM.  One row in four: 69 us; one in three would read
-// nearly every piece and gains nothing (dense again).
-constexpr int kSparse = 4;
+// A's 268 MB: 49 us, bound by DRAM.  From a cold L2 the two take 84 and 64, and one row
+// in four 76; one in three would read nearly every piece and gains nothing (dense again).
+// Where no warp has a second column, each waits for its chain of gathers: 12288 x 700
+// takes 66 us dense, 57 with one row in twelve and 85 with one in four, so the line is
+// one in eight there.
+constexpr int kSparse = 4, kSparseFew = 8;
+
+// The best of the block's columns from the rows with a dual alone (nz of them).  A function of its own: inlined beside it, the dense
+// pass's loop is scheduled worse (82 us instead of 66 at 12288 x 700).
+__device__ __noinline__ Best sparse_columns(int m, int nz, const double* __restrict__ A, int lda,
+                                            const double* __restrict__ c,
+                                            const int32_t* __restrict__ pos, int owned) {
+    extern __shared__ __align__(16) double ysh[];
+    __shared__ int wn[kThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int G = gridDim.x, me = (m + 1) & ~1;
+    double best_d = -DBL_MAX;
+    int best_j = -1;
+    // the rows with a dual, in increasing order: each warp counts and then writes
+    // those of its run of rows
+    uint16_t* nzi = reinterpret_cast<uint16_t*>(ysh + me);
+    const int run = ((m + nw - 1) / nw + 31) & ~31;
+    const int r0 = min(m, warp * run), r1 = min(m, r0 + run);
+    int mine = 0;
+    for (int k = r0; k < r1; k += 32)
+        mine += __popc(__ballot_sync(0xffffffffu, k + lane < r1 && nonzero(ysh[k + lane])));
+    __syncthreads();
+    if (lane == 0) wn[warp] = mine;
+    __syncthreads();
+    int at = 0;
+    for (int w = 0; w < warp; ++w) at += wn[w];
+    for (int k = r0; k < r1; k += 32) {
+        const bool in = k + lane < r1 && nonzero(ysh[k + lane]);
+        const unsigned bal = __ballot_sync(0xffffffffu, in);
+        if (in) nzi[at + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(k + lane);
+        at += __popc(bal);
+    }
+    __syncthreads();
+    // two columns per warp at a time, eight gathers in flight per lane
+    for (int l = warp; l < owned; l += 2 * nw) {
+        const int j0 = blockIdx.x + G * l, j1 = j0 + G * nw;
+        const bool in0 = pos[j0] < 0, in1 = l + nw < owned && pos[j1] < 0;
+        const double* c0 = A + (size_t)j0 * lda;
+        const double* c1 = A + (size_t)(in1 ? j1 : j0) * lda;
+        double a0 = 0.0, a1 = 0.0;
+#pragma unroll 8
+        for (int t = lane; t < nz; t += 32) {
+            const int i = nzi[t];
+            const double v = ysh[i], u0 = __ldg(c0 + i), u1 = __ldg(c1 + i);
+            a0 = fma(u0, v, a0);
+            a1 = fma(u1, v, a1);
+        }
+        const double d0 = c[j0] - warp_sum(a0);
+        if (in0 && better(d0, j0, best_d, best_j)) { best_d = d0; best_j = j0; }
+        if (in1) {  // (uniform over the warp)
+            const double d1 = c[j1] - warp_sum(a1);
+            if (better(d1, j1, best_d, best_j)) { best_d = d1; best_j = j1; }
+        }
+    }
+    return {best_d, best_j, 0};
+}
 
 // d_j = c_j - y^T a_j for nonbasic j (d_{n+i} = -y_i for slacks); the block
 // that finishes last writes the largest d_j > tol_d (exact ties to the
@@ -101,66 +164,31 @@ __global__ void __launch_bounds__(kThreads) k_price_static(int m, int n, const d
                                                            int32_t* q_out, double* dq_out, Scratch* sc) {
     extern __shared__ __align__(16) double ysh[];  // read as double2 below
     const int me = (m + 1) & ~1;
-    for (int k = threadIdx.x; k < me; k += blockDim.x) ysh[k] = k < m ? y[k] : 0.0;
-    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __shared__ int wn[kThreads / 32];
+    int duals = 0;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < me; k += blockDim.x) {
+        const double v = k < m ? y[k] : 0.0;
+        ysh[k] = v;
+        duals += nonzero(v);
+    }
+    duals = __reduce_add_sync(0xffffffffu, duals);
+    if (lane == 0) wn[warp] = duals;
+    __syncthreads();
+    int nz = 0;
+    for (int w = 0; w < nw; ++w) nz += wn[w];
     const int half = m >> 1;
     const double2* y2 = reinterpret_cast<const double2*>(ysh);
     double best_d = -DBL_MAX;
     int best_j = -1;
     const int G = gridDim.x;
     const int owned = (n - (int)blockIdx.x + G - 1) / G;
-    // The rows with a dual, in increasing order, when they are at most a quarter of
-    // all: each warp counts and then writes those of its run of rows.
-    const int cap = m / kSparse;
-    double* nzv = ysh + me;
-    int* nzi = reinterpret_cast<int*>(nzv + cap);
-    __shared__ int wn[kThreads / 32];
-    const int run = ((m + nw - 1) / nw + 31) & ~31;
-    const int r0 = min(m, warp * run), r1 = min(m, r0 + run);
-    int mine = 0;
-    for (int k = r0; k < r1; k += 32) mine += __popc(__ballot_sync(0xffffffffu, k + lane < r1 && ysh[k + lane] != 0.0));
-    if (lane == 0) wn[warp] = mine;
-    __syncthreads();
-    int nz = 0, at = 0;
-    for (int w = 0; w < nw; ++w) {
-        if (w == warp) at = nz;
-        nz += wn[w];
-    }
-    const bool sparse = nz <= cap;
+    const bool sparse = nz <= m / (owned > nw ? kSparse : kSparseFew);
     if (sparse) {
-        for (int k = r0; k < r1; k += 32) {
-            const double v = k + lane < r1 ? ysh[k + lane] : 0.0;
-            const unsigned bal = __ballot_sync(0xffffffffu, v != 0.0);
-            if (v != 0.0) {
-                const int e = at + __popc(bal & ((1u << lane) - 1u));
-                nzv[e] = v;
-                nzi[e] = k + lane;
-            }
-            at += __popc(bal);
-        }
-        __syncthreads();
-        // two columns per warp at a time, eight gathers in flight per lane
-        for (int l = warp; l < owned; l += 2 * nw) {
-            const int j0 = blockIdx.x + G * l, j1 = j0 + G * nw;
-            const bool in0 = pos[j0] < 0, in1 = l + nw < owned && pos[j1] < 0;
-            const double* c0 = A + (size_t)j0 * lda;
-            const double* c1 = A + (size_t)(in1 ? j1 : j0) * lda;
-            double a0 = 0.0, a1 = 0.0;
-#pragma unroll 4
-            for (int t = lane; t < nz; t += 32) {
-                const int i = nzi[t];
-                const double v = nzv[t], u0 = __ldg(c0 + i), u1 = __ldg(c1 + i);
-                a0 = fma(u0, v, a0);
-                a1 = fma(u1, v, a1);
-            }
-            const double d0 = c[j0] - warp_sum(a0);
-            if (in0 && better(d0, j0, best_d, best_j)) { best_d = d0; best_j = j0; }
-            if (in1) {  // (uniform over the warp)
-                const double d1 = c[j1] - warp_sum(a1);
-                if (better(d1, j1, best_d, best_j)) { best_d = d1; best_j = j1; }
-            }
-        }
+        const Best b = sparse_columns(m, nz, A, lda, c, pos, owned);
+        best_d = b.d;
+        best_j = b.j;
     }
     for (int l = warp; l < owned && !sparse; l += nw) {
         const int j = blockIdx.x + G * l;
@@ -209,9 +237,11 @@ __global__ void __launch_bounds__(kThreads) k_price_static(int m, int n, const d
     }
 }
 
-// y, and the list of its nonzeros
+// y, and the rows of its nonzeros: 8.5 m bytes, two blocks per SM up to the largest m (with
+// their values and 32-bit rows, 11 m bytes, one block above 10,400 rows: 12288 x 4096
+// took 171 us dense instead of 123)
 size_t price_smem(int m) {
-    return (size_t)((m + 1) & ~1) * sizeof(double) + (size_t)(m / kSparse) * (sizeof(double) + sizeof(int));
+    return (size_t)((m + 1) & ~1) * sizeof(double) + (size_t)(m / kSparse) * sizeof(uint16_t);
 }
 
 // Identity of the calling thread's current context (driver entry points
