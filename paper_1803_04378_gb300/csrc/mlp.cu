@@ -154,7 +154,8 @@ __global__ void __launch_bounds__(256) k_input16(const float* __restrict__ X, in
     pdl_enter();
     __shared__ __half tile[kTile][kTile + 2];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int c0 = blockIdx.x * kTile, r0 = blockIdx.y * kTile;
+    const int tc = (cols + kTile - 1) / kTile;  // tiles in a row of them: one grid dimension, for any batch
+    const int c0 = blockIdx.x % tc * kTile, r0 = blockIdx.x / tc * kTile;
 #pragma unroll
     for (int i = 0; i < kTile; i += 8) {
         const int r = r0 + ty + i, c = c0 + tx;
@@ -184,7 +185,8 @@ __global__ void __launch_bounds__(256) k_bce(const float* __restrict__ z, const 
     pdl_enter();
     __shared__ __half tile[kTile][kTile + 2];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int c0 = blockIdx.x * kTile, r0 = blockIdx.y * kTile;
+    const int tc = (cols + kTile - 1) / kTile;  // tiles in a row of them: one grid dimension, for any batch
+    const int c0 = blockIdx.x % tc * kTile, r0 = blockIdx.x / tc * kTile;
     const float inv = 1.f / (float)rows;
     float l = 0.f;
 #pragma unroll
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(256) k_bce(const float* __restrict__ z, const 
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w = 1; w < 8; ++w) l += wl[w];
-        part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = l;
+        part[blockIdx.x] = l;
     }
 #pragma unroll
     for (int i = 0; i < kTile; i += 8) {
@@ -424,6 +426,9 @@ int refresh_weights(lp_mlp* h, float lr = 0.f) {
     return LP_OK;
 }
 
+// 32 x 32 tiles of a batch's rows, padded to 64, by `cols` columns
+unsigned tiles(int cols, int B) { return (unsigned)((cols + kTile - 1) / kTile) * (unsigned)(pad64(B) / kTile); }
+
 // the hidden layers for a batch already in x16; back: what the backward pass reads is kept too
 int hidden_layers(lp_mlp* h, int B, bool back) {
     const float *b1 = h->p + h->off[1], *b2 = h->p + h->off[3];
@@ -443,7 +448,7 @@ int forward_backward(lp_mlp* h, int B, const float* t) {
     if ((rc = gemm(h, B, h->out, h->hid, h->a2, h->hid_p, h->w3t, h->hid_p,
                    EpiAct{h->p + h->off[5], h->z3, nullptr, nullptr, 0, 0, B, h->out})))
         return rc;
-    MCK(launch_k(k_bce, dim3((h->out + kTile - 1) / kTile, pad64(B) / kTile), dim3(256), 0, h->stream, true,
+    MCK(launch_k(k_bce, dim3(tiles(h->out, B)), dim3(256), 0, h->stream, true,
                  (const float*)h->z3, t, B, h->out, h->dz3, h->out_p, h->dz3T, h->b_p, h->part));
     if ((rc = gemm(h, B, h->hid, h->out, h->dz3, h->out_p, h->w3n, h->out_p,
                    EpiReluBack{h->z2, h->dz2, h->dz2T, h->hid_p, h->b_p, B, h->hid})))
@@ -460,14 +465,14 @@ int forward_backward(lp_mlp* h, int B, const float* t) {
         return rc;
     const ColSum q{{h->dz3, h->dz2, h->dz1}, {h->g + h->off[5], h->g + h->off[3], h->g + h->off[1]},
                    {h->out_p, h->hid_p, h->hid_p}, {h->out, h->hid, h->hid}, h->part,
-                   (h->out + kTile - 1) / kTile * (pad64(B) / kTile), h->loss};
+                   (int)tiles(h->out, B), h->loss};
     MCK(launch_k(k_colsum, dim3((std::max(h->out, h->hid) + kSumCols - 1) / kSumCols, 3), dim3(256), 0, h->stream, true, q, B));
     return LP_OK;
 }
 
 int load_x(lp_mlp* h, const float* X, int B, bool back) {
     if (B < 1 || B > h->maxb || !X) return LP_ERR_INVALID_ARG;
-    MCK(launch_k(k_input16, dim3((h->in + kTile - 1) / kTile, pad64(B) / kTile), dim3(256), 0, h->stream, false, X,
+    MCK(launch_k(k_input16, dim3(tiles(h->in, B)), dim3(256), 0, h->stream, false, X,
                  B, h->in, h->x16, h->in_p, back ? h->xT : (__half*)nullptr, h->b_p));
     return LP_OK;
 }
