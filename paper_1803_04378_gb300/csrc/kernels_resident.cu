@@ -70,7 +70,7 @@ constexpr int kRThreads = 512;
 constexpr int kRWarps = kRThreads / 32;
 constexpr int kRPrice = 8;        // warps that screen and poll; the others apply the rank-1 update
 constexpr int kRMail = kRWarps - 1;  // the warp that fences for the CTA and sends what publishes its data
-constexpr int kRMaxCtas = 32 * kRPrice;
+constexpr int kRMaxCtas = 32 * (kRPrice - 1);  // a pricing warp that does not poll moves the slots of A
 constexpr int kRChunks = 4;       // 16-byte chunks of a record: three payload words and the stamp
 constexpr int kRWords = 3 * kRChunks;
 constexpr unsigned kRMore = 1u << 31;  // PRICE record: more than one column listed
@@ -873,7 +873,6 @@ __global__ void __launch_bounds__(kRThreads, 1) k_iterate_r(DevState s, int iter
             // the others, and the pricing warps that do not poll: the pivot's moves and update
             if (piv && warp >= nwu) {
                 if (warp < kRPrice) move_rows(tid - 32 * nwu, 32 * (kRPrice - nwu));
-                else if (nwu == kRPrice) move_rows(tid - 32 * kRPrice, kRThreads - 32 * kRPrice);
                 apply_rows(r);
             }
             __syncthreads();
