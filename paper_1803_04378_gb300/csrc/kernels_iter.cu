@@ -692,8 +692,8 @@ size_t price_smem_bytes(int ld) { return (size_t)ld * sizeof(double); }
 size_t update_smem_bytes(int ld) { return 2 * (size_t)ld * sizeof(double); }
 
 void configure_iter_kernels() {
-    raise_smem_limit(reinterpret_cast<const void*>(k_price));
-    raise_smem_limit(reinterpret_cast<const void*>(k_update));
+    raise_smem_limit<k_price>();
+    raise_smem_limit<k_update>();
 }
 
 void launch_init_slack(const DevState& s, cudaStream_t st) {
@@ -727,8 +727,8 @@ int occupancy_price(int ld) {
 size_t iterate_smem_bytes(int ld) { return 2 * (size_t)ld * sizeof(double); }
 
 int occupancy_iterate(int ld) {
-    raise_smem_limit(reinterpret_cast<const void*>(k_iterate<false>));
-    raise_smem_limit(reinterpret_cast<const void*>(k_iterate<true>));
+    raise_smem_limit<k_iterate<false>>();
+    raise_smem_limit<k_iterate<true>>();
     int nb = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_iterate<false>, kUpdateThreads, iterate_smem_bytes(ld));
     return nb;

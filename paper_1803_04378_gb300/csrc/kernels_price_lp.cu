@@ -256,7 +256,7 @@ void launch_price_lp(const DevState& s, const Geometry& g, cudaStream_t st, bool
 
 int occupancy_price_lp(int ld) {
     const size_t smem = (size_t)ld * (sizeof(float) + sizeof(double));
-    raise_smem_limit(reinterpret_cast<const void*>(k_price_lp));
+    raise_smem_limit<k_price_lp>();
     int nb = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_price_lp, kLpThreads, smem);
     return nb;

@@ -1293,17 +1293,21 @@ unsigned resident_meetings(int iters) { return kRStepMeetings * (unsigned)iters 
 size_t resident_meet_bytes(int ctas) { return sizeof(ulonglong2) * 2 * kRChunks * (size_t)ctas * ctas; }
 
 cudaError_t resident_room(size_t* room) {
-    const ResKernel k[3] = {res_kernel(true, true), res_kernel(true, false), res_kernel(false, false)};
-    *room = SIZE_MAX;
-    for (ResKernel f : k) {
-        size_t r = 0;
-        const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(f), &r);
-        if (e != cudaSuccess) return e;
-        *room = std::min(*room, r);
-    }
-    return cudaSuccess;
+    size_t r[3] = {};
+    cudaError_t e = raise_smem_limit<k_iterate_r<true, true>>(&r[0]);
+    if (e == cudaSuccess) e = raise_smem_limit<k_iterate_r<true, false>>(&r[1]);
+    if (e == cudaSuccess) e = raise_smem_limit<k_iterate_r<false, false>>(&r[2]);
+    *room = std::min(r[0], std::min(r[1], r[2]));
+    return e;
 }
 
+// The layouts in order: A and B^-1 in shared memory, A alone, neither.  Each is faster
+// than k_iterate_s wherever it is the one that fits (us per pivot, k live rows):
+//   both     4096 x 8192, k = 300   17.9 / 32.5;  5500 x 11000, k = 200    22 / 38
+//   A alone  4096 x 8192, k = 500   22.1 / 36.3;  k = 700    28.5 / 41.8;
+//            5500 x 11000, k = 500  30 / 49;      1800 x 2000, k = 1000  22.3 / 31.8
+//   neither  4096 x 8192, k = 1000  37.7 / 50.4;  k = 2000   78.7 / 86.5;
+//            5500 x 11000, k = 900  52 / 70;      k = 2500  141 / 150;  120 x 70000  16.5 / 29.6
 bool resident_plan(int m, int n, int ld, int ctas, int k_live, int iters, size_t room, ResidentPlan* out) {
     // room for every pivot of the launch to add a live slot, and at least one
     const int want = std::min(ld, (k_live + iters + 1 + 63) & ~63);

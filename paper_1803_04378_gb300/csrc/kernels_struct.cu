@@ -1203,7 +1203,7 @@ bool struct_engine_fits(int m, int ld, int ctas) {
 }
 
 int occupancy_iterate_s(int ld) {
-    raise_smem_limit(reinterpret_cast<const void*>(k_iterate_s));
+    raise_smem_limit<k_iterate_s>();
     int nb = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_iterate_s, kUpdateThreads, iterate_s_smem_bytes(ld));
     return nb;

@@ -15,6 +15,7 @@
 //          device, so a captured graph of many iterations needs no host
 //          round trip.
 #pragma once
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -274,16 +275,21 @@ inline cudaError_t launch_k(void (*kernel)(Args...), dim3 grid, dim3 block, size
 // thread's between this setting and the launch, would have the launch refused.
 // Set to the same value by all, it is safe from any thread; a launch still gets
 // what it asks for and no more.
-inline cudaError_t raise_smem_limit(const void* kernel, size_t* room = nullptr) {
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-    int dev = 0, optin = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+template <auto kKernel>
+cudaError_t raise_smem_limit(size_t* room = nullptr) {
+    static std::atomic<int> fixed{-1};  // its static part, asked for once: a property of the code
+    const void* kernel = reinterpret_cast<const void*>(kKernel);
+    int dev = 0, optin = 0, st = fixed.load(std::memory_order_relaxed);
+    cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess && st < 0) {
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, kernel);
+        if (e == cudaSuccess) fixed.store(st = (int)fa.sharedSizeBytes, std::memory_order_relaxed);
+    }
     if (e != cudaSuccess) return e;
-    const int most = optin - (int)fa.sharedSizeBytes;
-    if (room) *room = (size_t)most;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (room) *room = (size_t)(optin - st);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - st);
 }
 
 struct Geometry {

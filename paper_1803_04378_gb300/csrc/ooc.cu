@@ -204,7 +204,7 @@ void launch_ooc_fetch_row(const DevState& s, const double* host_binv, const doub
 }
 
 int configure_ooc_kernels() {
-    return raise_smem_limit(reinterpret_cast<const void*>(k_ooc_update)) == cudaSuccess ? 0 : -1;
+    return raise_smem_limit<k_ooc_update>() == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace lpgb
