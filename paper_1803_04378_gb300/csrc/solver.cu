@@ -104,7 +104,7 @@ int cuda_fail(cudaError_t e) {
 // larger ones get an allocation of their own.  A handle makes a dozen
 // cudaMalloc calls (and its destruction as many cudaFree calls) instead of
 // dozens.  Everything is freed with the handle (free_all).
-constexpr size_t kPoolMax = size_t(1) << 20, kPoolChunk = size_t(16) << 20, kPoolAlign = 256;
+constexpr size_t kPoolMax = size_t(4) << 20, kPoolChunk = size_t(16) << 20, kPoolAlign = 256;
 template <typename T>
 int dalloc(lp_handle* h, T** ptr, size_t count) {
     const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
