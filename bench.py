@@ -482,8 +482,9 @@ def main():
             "frac": (kflops / kt / 1e12 / FP64_PEAK_TFLOPS) if kt else None,
             "peak_source": "nominal FP64 rate (2 FMA per clock per SM x 152 SMs x 2.07 GHz), no measured FP64 peak"}
     if kname == "k_iterate_r":
-        # the live rows of A and columns of B^-1 stay in L2 across pivots: the
-        # bound is the FP64 pipe, and the HBM figure is given beside it
+        # the live rows of A and columns of B^-1 stay in shared memory (where they fit,
+        # else in L2) across pivots: the bound is the FP64 pipe, and the HBM figure
+        # is given beside it
         roofline = dict(bound="alu", kernel=kname, **fp64, hbm=hbm)
     else:
         roofline = dict(bound="hbm", kernel=kname, **hbm, fp64=fp64)
@@ -626,7 +627,7 @@ def main():
                        "step": "one full solve from the slack basis to optimality",
                        "l2": ("no flush: the inputs (A 268 MB, its slot-ordered copy 268 MB, B^-1 134 MB) exceed "
                               "L2 and every step's reset rebuilds the slot-ordered copy; within a solve the "
-                              "structured engine keeps its live rows and columns L2-resident by design"
+                              "structured engine keeps its live rows and columns on the chip by design"
                               if results[0].persistent == 2 else
                               "no flush: A (268 MB) + B^-1 (134 MB) streamed every pivot exceed L2"),
                        "engine": {2: "slack-structured persistent", 1: "dense persistent",

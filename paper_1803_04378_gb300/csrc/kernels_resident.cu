@@ -4,8 +4,8 @@
 // The method, the slot layout and the arithmetic are those of k_iterate_s
 // (kernels_struct.cu): PRICE over the k live rows, FTRAN and the rank-1 update
 // over the k live columns of B^-1, slot moves, the same order of every sum --
-// so the pivots, B^-1, bbar and y are bit-identical to it.  What differs is
-// where the operands live and how the CTAs meet.
+// so the pivots, B^-1, bbar and y are bit-identical to it (-0 and 0 as one value).
+// What differs is where the operands live and how the CTAs meet.
 //
 // Residence.  CTA b owns the columns j = b, b + G, ... of A and the rows
 // i = b, b + G, ... of B^-1.  Their live parts stay in shared memory for the
@@ -30,8 +30,9 @@
 // each of the record's stores costs 0.9 to 1.3 us a pivot, a fence in every polling
 // warp 0 to 0.5, this 0 to 0.18.)  So do the repair's meeting and those without a record.
 // The PRICE meeting publishes nothing.  After it the pivot row's owner overwrites the
-// row, which every CTA has read: each record sent is computed from the row's
-// values, so a read that returned the later ones would be the cause of itself.
+// row, which every CTA has read: each sends its record on a condition over all of the
+// row's values (the range of the new y), so a read that returned the later ones would
+// be the cause of itself.
 //
 // PRICE decides on intervals.  The FP32 screen gives every column an interval
 // that holds its reduced cost.  The record of a CTA is its largest lower end
@@ -49,11 +50,11 @@
 //
 // What bounds it: latency.  A pivot is a chain of two meetings, two L2
 // round trips (pivot row, entering column; 0.6 us each), seven block barriers and
-// the reductions between them; of 17.0 us at 4096 x 8192 the FP64 pipe needs 2.6 us for
+// the reductions between them; of 17.2 us at 4096 x 8192 the FP64 pipe needs 2.6 us for
 // FTRAN, and 2.5 us for the update that PRICE hides.  Against k_iterate_s, whose
-// operands stay in L2 and whose 1024-thread CTAs meet through atomics: 30.1 -> 17.0 us
+// operands stay in L2 and whose 1024-thread CTAs meet through atomics: 30.1 -> 17.2 us
 // per pivot at 4096 x 8192, 19.8 -> 9.0 at 701 x 1203, 20.6 -> 9.0 at 200 x 300,
-// 24.3 -> 9.1 on a degenerate 256 x 512 under the safety net.
+// 24.3 -> 9.05 on a degenerate 256 x 512 under the safety net.
 #include "lpgb_internal.cuh"
 #include "struct_common.cuh"
 #include "../../include/lpgb.h"
@@ -99,7 +100,7 @@ __device__ __forceinline__ ulonglong2 ld_acquire_b128(const ulonglong2* p) {
 // One chunk of the CTA's record under `seq`, into CTA dest's mailbox.  Every CTA has a
 // mailbox of its own, which no other polls, a sender's 16 bytes beside the next
 // sender's: a warp polls 32 senders in four lines.  One record for all, 64 bytes apart
-// and polled by every CTA, held up its writer (17.9 us a pivot against 17.0 at
+// and polled by every CTA, held up its writer (17.9 us a pivot against 17.0 then at
 // 4096 x 8192 on 152 CTAs, 10.6 against 9.5 at 1024 x 2048); chunks of several CTAs in
 // one line that all poll took 2.3 us a meeting.
 __device__ __forceinline__ void meet_put(ulonglong2* buf, unsigned seq, int dest, int chunk, unsigned a, unsigned b,
