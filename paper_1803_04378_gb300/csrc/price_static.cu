@@ -96,8 +96,9 @@ __device__ void block_best(double& d, int& j) {
 // in four 76; one in three would read nearly every piece and gains nothing (dense again).
 // Where no warp has a second column, each waits for its chain of gathers: 12288 x 700
 // takes 66 us dense, 57 with one row in twelve and 85 with one in four, so the line is
-// one in eight there.
-constexpr int kSparse = 4, kSparseFew = 8;
+// one in eight there.  Below kSparseMin rows there is nothing to gain, and the duals are
+// not even counted (100 x 200, its memset included: 10.4 us, 11.1 with the list).
+constexpr int kSparse = 4, kSparseFew = 8, kSparseMin = 512;
 
 // The best of the block's columns from the rows with a dual alone (nz of them).  A function of its own: inlined beside it, the dense
 // pass's loop is scheduled worse (82 us instead of 66 at 12288 x 700).
@@ -157,6 +158,8 @@ __device__ __noinline__ Best sparse_columns(int m, int nz, const double* __restr
 // d_j = c_j - y^T a_j for nonbasic j (d_{n+i} = -y_i for slacks); the block
 // that finishes last writes the largest d_j > tol_d (exact ties to the
 // smallest j) to q_out / dq_out, or q_out = -1 when none exceeds tol_d.
+// kList: m >= kSparseMin.
+template <bool kList>
 __global__ void __launch_bounds__(kThreads) k_price_static(int m, int n, const double* __restrict__ A, int lda,
                                                            const double* __restrict__ c,
                                                            const double* __restrict__ y,
@@ -171,20 +174,23 @@ __global__ void __launch_bounds__(kThreads) k_price_static(int m, int n, const d
     for (int k = threadIdx.x; k < me; k += blockDim.x) {
         const double v = k < m ? y[k] : 0.0;
         ysh[k] = v;
-        duals += nonzero(v);
+        if (kList) duals += nonzero(v);
     }
-    duals = __reduce_add_sync(0xffffffffu, duals);
-    if (lane == 0) wn[warp] = duals;
+    if (kList) {
+        duals = __reduce_add_sync(0xffffffffu, duals);
+        if (lane == 0) wn[warp] = duals;
+    }
     __syncthreads();
     int nz = 0;
-    for (int w = 0; w < nw; ++w) nz += wn[w];
+    if (kList)
+        for (int w = 0; w < nw; ++w) nz += wn[w];
     const int half = m >> 1;
     const double2* y2 = reinterpret_cast<const double2*>(ysh);
     double best_d = -DBL_MAX;
     int best_j = -1;
     const int G = gridDim.x;
     const int owned = (n - (int)blockIdx.x + G - 1) / G;
-    const bool sparse = nz <= m / (owned > nw ? kSparse : kSparseFew);
+    const bool sparse = kList && nz <= m / (owned > nw ? kSparse : kSparseFew);
     if (sparse) {
         const Best b = sparse_columns(m, nz, A, lda, c, pos, owned);
         best_d = b.d;
@@ -281,7 +287,7 @@ int setup_device(int dev, DeviceSetup** out) {
     if (!s.ready) {
         void* ptr = nullptr;
         if (cudaGetSymbolAddress(&ptr, g_price_scratch) != cudaSuccess || ptr == nullptr) return LP_ERR_CUDA;
-        if (cudaFuncSetAttribute(k_price_static, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(k_price_static<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)price_smem(LP_PRICE_STATIC_MAX_M)) != cudaSuccess)
             return LP_ERR_CUDA;
         int sms = 0;
@@ -317,8 +323,8 @@ extern "C" int lp_price_static(int32_t m, int32_t n, const double* A_colmajor, i
     if (blocks > n) blocks = n;
     if (cudaMemsetAsync(&s->scratch->ticket, 0, sizeof(int32_t), st) != cudaSuccess) return LP_ERR_CUDA;
     const size_t smem = price_smem(m);
-    k_price_static<<<blocks, kThreads, smem, st>>>(m, n, A_colmajor, lda, c, y, pos, tol_d, q_out, dq_out,
-                                                   s->scratch);
+    const auto kernel = m >= kSparseMin ? k_price_static<true> : k_price_static<false>;
+    kernel<<<blocks, kThreads, smem, st>>>(m, n, A_colmajor, lda, c, y, pos, tol_d, q_out, dq_out, s->scratch);
     if (cudaGetLastError() != cudaSuccess) return LP_ERR_CUDA;
     return LP_OK;
 }

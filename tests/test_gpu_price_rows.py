@@ -1,5 +1,5 @@
 """lp_price_static around the list of the rows with a dual: the largest m (two blocks share
-an SM's shared memory), list lengths at the lines between the two passes (m / 4 where
+an SM's shared memory), the smallest m with a list, list lengths at the lines between the two passes (m / 4 where
 warps have several columns, m / 8 where none has a second), runs of rows that end
 inside a warp's 32, signed zeros and NaN among the duals.
 
@@ -38,7 +38,7 @@ def _price(m, n, k, seed, special=False):
 
 
 @pytest.mark.parametrize("n", [3, 700, 9000])
-@pytest.mark.parametrize("m", [12288, 12287, 10401, 513, 33, 7])
+@pytest.mark.parametrize("m", [12288, 12287, 10401, 513, 512, 511, 33, 7])
 @pytest.mark.parametrize("part", [4, 8])
 def test_both_sides_of_the_lines(m, n, part):
     for k in (m // part, min(m, m // part + 1)):
